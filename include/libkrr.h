@@ -456,7 +456,7 @@ krr_status krr_tune_load(krr_handle h, const char* path);
  * row-major), Q and Y (N x m column-major) with N <= 16384, d <= 8 and
  * m <= 16.  Larger problems return KRR_ERR_SIZE_LIMIT; host arrays and bad
  * values return KRR_ERR_INVALID_ARG.
- * It allocates nothing.  Its scratch is one fixed device array of 10,415,872
+ * It allocates nothing.  Its scratch is one fixed device array of 10,210,816
  * bytes, held by every GPU that loads the library until the process exits;
  * an internal request beyond a region of it returns KRR_ERR_OOM instead of
  * allocating.  The first call made with a device current looks up that

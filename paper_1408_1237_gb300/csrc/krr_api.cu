@@ -122,6 +122,7 @@ cudaError_t sub_context(Ctx& c, size_t k, Ctx** out) {
     if (!s) return cudaErrorMemoryAllocation;
     s->device = c.device;
     s->num_sms = c.num_sms;
+    s->h_counts = c.h_counts;  // a preparation waits for its counts, so the words can be shared
     cudaError_t e = cudaMalloc(&s->d_err, sizeof(int));
     if (!e) e = cudaMemset(s->d_err, 0, sizeof(int));
     if (e) {
@@ -281,6 +282,7 @@ krr_status krr_create(krr_handle* out) {
   if (!e) e = cudaMalloc(&c.d_err, sizeof(int));
   if (!e) e = cudaMemset(c.d_err, 0, sizeof(int));
   if (!e) e = cudaMallocHost(&c.h_status, 64 * sizeof(int));
+  if (!e) c.h_counts = c.h_status + 32;
   if (!e) e = cudaEventCreate(&c.ev0);
   if (!e) e = cudaEventCreate(&c.ev1);
   if (!e) e = cudaStreamCreateWithFlags(&c.work, cudaStreamNonBlocking);
@@ -547,7 +549,9 @@ krr_status krr_points_create(krr_handle h, const float* X, int64_t N, int d, flo
   copy_product_options(pc, c);
   cudaError_t e = cudaMalloc(&pc.d_err, sizeof(int));
   if (!e) e = cudaMemsetAsync(pc.d_err, 0, sizeof(int), st);
+  pc.h_counts = c.h_counts;  // the handle's pinned words, for this one wait
   if (!e) e = prepare_points(pc, dX, N, d, sigma, "points", pts->P, st);  // waits once
+  pc.h_counts = nullptr;
   if (e) {
     free_points(pts);
     return cuda_error(c, e, fn);

@@ -51,7 +51,6 @@ constexpr int NA_MAX_DEV = 64;
 // Upper bounds of every buffer the prep and product code requests for
 // N <= NA_MAX_N, d <= NA_MAX_D, m <= NA_MAX_M (see prep.cu and mvp.cu).
 constexpr int64_t NPAD = NA_MAX_N;                 // multiple of PAD
-constexpr int64_t NCHUNK = NA_MAX_N / 2048;         // radix-sort chunks
 constexpr int64_t NBLK = NA_MAX_N / 32;             // warp blocks (T >= 1)
 constexpr int64_t NTILE = NPAD / 256;               // source tiles
 constexpr int64_t MAX_SPLITS = 64;
@@ -65,12 +64,7 @@ constexpr Region kRegions[] = {
     {"na.xs", sizeof(float) * NPAD * NA_MAX_D},
     {"na.perm", sizeof(int) * NPAD},
     {"sort.ka", sizeof(uint32_t) * NA_MAX_N},
-    {"sort.kb", sizeof(uint32_t) * NA_MAX_N},
-    {"sort.va", sizeof(int) * NA_MAX_N},
-    {"sort.vb", sizeof(int) * NA_MAX_N},
-    {"sort.hist", sizeof(uint32_t) * 256 * NCHUNK},
     {"sort.bbp", sizeof(float) * 2 * NA_MAX_D * 256},
-    {"sort.bb", sizeof(float) * 2 * NA_MAX_D},
     {"na.ctr", sizeof(float) * NBLK * NA_MAX_D},
     {"na.order", sizeof(int) * NBLK},
     {"na.nexp", sizeof(int)},
@@ -101,9 +95,9 @@ constexpr size_t total_bytes() {
 
 #define KRR_NOALLOC_SCRATCH_BYTES (krr::total_bytes())
 
-// The scratch array: 10,415,872 bytes (about 10 MB).  Host code must not take its address
+// The scratch array: 10,210,816 bytes (about 10 MB).  Host code must not take its address
 // directly: use the pointer from cudaGetSymbolAddress.
-static_assert(KRR_NOALLOC_SCRATCH_BYTES == 10415872, "the documented scratch size");
+static_assert(KRR_NOALLOC_SCRATCH_BYTES == 10210816, "the documented scratch size");
 static __device__ __align__(256) unsigned char g_noalloc_scratch[KRR_NOALLOC_SCRATCH_BYTES];
 
 namespace krr {
