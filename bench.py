@@ -4,7 +4,7 @@ time-to-solution (the two halves of the headline metric).
 
 One JSON line on rank 0.  A step is one full kernel product y = (K_hat +
 gamma I) q through the C ABI on the 2^20-point unit-cube cloud (d = 3,
-sigma 0.05, gamma 1e-3): point preparation (Morton sort, packing, block
+sigma 0.05, gamma 1e-3): point preparation (Hilbert sort, packing, block
 metadata), the product kernel and its finalize.  `value` is whole-job
 Gpairs/s (N^2 pairs per step per rank, all ranks, over the slowest rank's
 device time).  Extra keys report the 16-column product, the roofline of the
@@ -249,7 +249,7 @@ def bench_config(world):
     return {
         "workload": f"gaussian kernel product y=(K_hat+gamma I)q, N={MVP_N} uniform "
                     "unit cube d=3, sigma=0.05, gamma=1e-3, q~N(0,1), m=1; step = "
-                    "prep (Morton sort, pack) + product + finalize through the C ABI",
+                    "prep (Hilbert sort, pack) + product + finalize through the C ABI",
         "l2": "512 MB buffer written between timed steps (inputs are 16 MB)",
         "parallelism": f"{world} independent problems (one per GPU)",
     }

@@ -180,7 +180,7 @@ typedef enum {
     /* Target-row shard emulation (the row partition a multi-GPU product
      * would use, run on one GPU): with SHARD_COUNT = P > 1, krr_kernel_mvp
      * on this handle computes and writes only shard SHARD_INDEX = k of its
-     * target rows: the sorted (Morton-order) super-blocks
+     * target rows: the sorted (Hilbert-order) super-blocks
      * [k nsb / P, (k+1) nsb / P) of 256 targets, that is 1/P of the work.
      * The other rows of Y are left as they were (a host Y is uploaded
      * first).  The plans are those of the whole product, so the P shards
@@ -231,7 +231,7 @@ krr_status krr_set_option(krr_handle h, int option, int value);
  * prec: KRR_FP32 (max relative error per element, against the FP64 sum
  * scaled by sum_j |Q_jc| K_hat_ij + gamma |Q_ic|, below 1e-5) or KRR_BF16 /
  * KRR_FP16 (reduced-precision kernel values, float32 accumulation).
- * The call waits briefly for the point preparation (Morton sort and block
+ * The call waits briefly for the point preparation (Hilbert sort and block
  * metadata) to read the block counts that size the product grids; the
  * product itself is asynchronous on device arrays. */
 krr_status krr_kernel_mvp(krr_handle h, const float* X, int64_t N, int d,
@@ -240,7 +240,7 @@ krr_status krr_kernel_mvp(krr_handle h, const float* X, int64_t N, int d,
 
 /* ----------------------------------------------------------- prepared point sets
  * Repeated products over one point set (a serving loop, a caller's own
- * iterative method, many weight vectors): the Morton sort, packing and block
+ * iterative method, many weight vectors): the Hilbert sort, packing and block
  * metadata of krr_kernel_mvp are done once, and each product then runs with
  * no host synchronisation, so it can be captured in a CUDA graph.
  *

@@ -246,10 +246,11 @@ cudaError_t sub_context(Ctx& c, size_t k, Ctx** out);
 void release_context(Ctx& c);
 
 // ---- prep.cu
-// Sort X (N x d row-major, device) along a Morton curve and pack the scaled,
+// Sort X (N x d row-major, device) along a Hilbert curve and pack the scaled,
 // tile-blocked structure-of-arrays copy.  `tag` names the workspace slots.
+// hilbert = false: Morton order.
 cudaError_t prepare_points(Ctx& c, const float* X, int64_t N, int d, float sigma,
-                           const char* tag, PointsDev& P, cudaStream_t st);
+                           const char* tag, PointsDev& P, cudaStream_t st, bool hilbert = true);
 // out[i] = in[perm[i]] (float columns, m of them, column stride N / Npad);
 // padded tail of each column set to zero.
 cudaError_t gather_sorted(const float* in, int64_t N, int m, const int* perm, int64_t Npad,

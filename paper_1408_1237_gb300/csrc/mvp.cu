@@ -3,7 +3,7 @@
 //   y_i = sum_j q_j exp(-|x_i - x_j|^2 / (2 sigma^2)) + shift q_i
 //
 // (Eqs. 1-3; the weighted kernel sum of Sec. 3.1, computed on the fly in O(N)
-// memory).  Points arrive prepared by prep.cu: Morton-sorted, unscaled; with
+// memory).  Points arrive prepared by prep.cu: Hilbert-sorted, unscaled; with
 // s = sqrt(log2(e) / (2 sigma^2)) a kernel value is 2^(-s^2 |x_i - x_j|^2).
 //
 // Kernel design:
