@@ -124,6 +124,8 @@ struct Ctx {
   // kernel values on the CUDA cores, the weighted sum on the tensor cores
   // (mvp_dirtc_kernel); false: the all-CUDA-core kernel mvp_dirm_kernel
   bool direct_tensor = true;
+  // sort points in Morton order (set while krr_mll_grad runs)
+  bool morton = false;
   // kernel function of every product and solve (KRR_KERNEL_*, krr_set_option)
   int kernel_family = 0;
   // autotuning of the products' source splits (KRR_OPT_AUTOTUNE): the first
@@ -248,9 +250,9 @@ void release_context(Ctx& c);
 // ---- prep.cu
 // Sort X (N x d row-major, device) along a Hilbert curve and pack the scaled,
 // tile-blocked structure-of-arrays copy.  `tag` names the workspace slots.
-// hilbert = false: Morton order.
+// Under c.morton they are sorted in Morton order.
 cudaError_t prepare_points(Ctx& c, const float* X, int64_t N, int d, float sigma,
-                           const char* tag, PointsDev& P, cudaStream_t st, bool hilbert = true);
+                           const char* tag, PointsDev& P, cudaStream_t st);
 // out[i] = in[perm[i]] (float columns, m of them, column stride N / Npad);
 // padded tail of each column set to zero.
 cudaError_t gather_sorted(const float* in, int64_t N, int m, const int* perm, int64_t Npad,

@@ -338,6 +338,16 @@ extern "C" krr_status krr_mll_grad(krr_handle h, const float* X, int64_t N, int 
   }
   if (!y) return set_error(c, KRR_ERR_INVALID_ARG, "%s: y is NULL", fn);
   cudaStream_t st = (cudaStream_t)stream;
+  // Morton order for the solves and the adjoint sums: dL/dlog sigma cancels by
+  // 1e4 and more, so another order of the points would move it by 1e-5 of its
+  // value at random (through the sums, and by 1e-6 through the last bits of
+  // the solutions); the adjoint takes the direct form for every pair, so the
+  // order costs it nothing
+  struct Order {
+    Ctx& c;
+    explicit Order(Ctx& cc) : c(cc) { c.morton = true; }
+    ~Order() { c.morton = false; }
+  } order(c);
   const int P = n_probes, nrhs = 1 + P, ncols = 2 * P + 1;
   float *dXin, *dy, *ddX = nullptr;
   bool sX, sy, sdX = false;
@@ -360,10 +370,7 @@ extern "C" krr_status krr_mll_grad(krr_handle h, const float* X, int64_t N, int 
   if (ss != KRR_OK && ss != KRR_NOT_CONVERGED) return ss;
   // adjoint sums
   PointsDev Pt;
-  // Morton order: the adjoint takes the direct form for every pair, so the
-  // order costs it nothing, and dL/dlog sigma cancels by 1e4 and more, so
-  // another summation order would move it by 1e-5 of its value at random
-  if ((e = prepare_points(c, dXin, N, d, sigma, "mll.pts", Pt, st, false))) return cuda_error(c, e, fn);
+  if ((e = prepare_points(c, dXin, N, d, sigma, "mll.pts", Pt, st))) return cuda_error(c, e, fn);
   const int ntiles = (int)(Pt.Npad / TS);
   const int64_t ctas = (N + ADJ_NT - 1) / ADJ_NT;
   int splits = (int)std::min<int64_t>(ntiles, std::max<int64_t>(1, (2LL * c.num_sms + ctas - 1) / ctas));

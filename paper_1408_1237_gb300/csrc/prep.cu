@@ -150,8 +150,9 @@ __global__ void __launch_bounds__(256)
 // (warp, item, lane); cnt holds 256 counters per warp.  The rank of item i is
 // the element's rank among its warp's equal digits; after a barrier the
 // caller scans the counters over the warps.  Elements whose bit of `valid` is
-// clear are left out.  A warp ranks 32 elements per step by one match of their
-// digits; put(i, rank) takes the results.
+// clear are left out.  A warp ranks 32 elements per step: the lanes with equal
+// digits come from 8 ballots (one match instruction took 24 us per pass at 16
+// items); put(i, rank) takes the results.
 template <int ITEMS, typename Put>
 __device__ __forceinline__ void warp_digit_ranks(const uint32_t (&key)[ITEMS], uint32_t valid, int shift,
                                                  uint32_t* cnt, Put put) {
@@ -159,8 +160,14 @@ __device__ __forceinline__ void warp_digit_ranks(const uint32_t (&key)[ITEMS], u
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
     const bool v = (valid >> i) & 1u;
-    const uint32_t digit = v ? (key[i] >> shift) & 0xFFu : 0x100u;
-    const uint32_t peers = __match_any_sync(0xffffffffu, digit);
+    const uint32_t digit = (key[i] >> shift) & 0xFFu;
+    uint32_t peers = __ballot_sync(0xffffffffu, v);
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      const bool set = (digit >> b) & 1u;
+      const uint32_t have = __ballot_sync(0xffffffffu, set);
+      peers &= set ? have : ~have;
+    }
     const uint32_t below = __popc(peers & ((1u << lane) - 1u));
     uint32_t base = 0;
     if (v) base = cnt[digit];
@@ -196,12 +203,14 @@ __device__ __forceinline__ uint32_t scan256(uint32_t v, uint32_t* ws) {
 
 // ---- cluster sort: the whole stable LSD radix sort of N <= CL_MAX_N keys in
 // one launch.  The elements live in the shared memory of CL_SIZE CTAs (position
-// p in CTA p / E, slot p % E, E = ITEMS * CL_THREADS); each 8-bit pass ranks
-// them in registers, exchanges the CTAs' digit counts and scatters the (key,
-// value) pairs through distributed shared memory.  Two cluster barriers per
-// pass replace three launches and a single-block scan, whose 4 x 46 us of
-// kernels at 50,000 points were latency: the product over 4096 points went
-// from 293 to 72 us, over 50,021 from 729 to 539 us.
+// p in CTA p / E, slot p % E, E = ITEMS * CL_THREADS); each 8-bit pass sorts a
+// CTA's elements by digit in its own shared memory, exchanges the CTAs' digit
+// counts and writes the digit runs to their places through distributed shared
+// memory.  Two cluster barriers per pass replace three launches and a
+// single-block scan, whose 4 x 46 us of kernels at 50,000 points were latency:
+// the product over 4096 points went from 293 to 72 us, over 50,021 from 729
+// to 539 us.  (Without the local sort every lane of a remote store has its
+// own target row: the sort took 51 us at 50,021 points and 113 us at 131,072.)
 template <int ITEMS>
 constexpr size_t cluster_sort_smem() {
   return (size_t)ITEMS * CL_THREADS * 8 + (CL_THREADS / 32) * 256 * 4;
@@ -252,18 +261,34 @@ __global__ void __launch_bounds__(CL_THREADS, 1)
     for (int e = 0; e < 8; ++e) wc[lane + 32 * e] = 0u;
     __syncwarp();
     warp_digit_ranks<ITEMS>(key, valid, shift, wc, [&](int i, uint32_t r) { vr[i] |= r << 17; });
-    __syncthreads();
+    __syncthreads();  // counters complete; every element of this CTA is in registers
+    uint32_t total = 0;
     if (tid < 256) {
-      uint32_t run = 0;
 #pragma unroll 8
       for (int w = 0; w < CL_THREADS / 32; ++w) {
         const uint32_t c = cnt[w * 256 + tid];
-        cnt[w * 256 + tid] = run;
-        run += c;
+        cnt[w * 256 + tid] = total;
+        total += c;
       }
-      ctot[tid] = run;
+      ctot[tid] = total;
     }
-    cluster_barrier();  // counts published; every element of this pass is in registers
+    const uint32_t start = scan256(total, ws);  // this CTA's first slot of the digit
+    if (tid < 256) off[tid] = start;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+      if (!((valid >> i) & 1u)) continue;
+      const uint32_t digit = (key[i] >> shift) & 0xFFu;
+      sbuf[off[digit] + wc[digit] + (vr[i] >> 17)] = make_uint2(key[i], vr[i] & 0x1FFFFu);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+      const uint2 kv = sbuf[warp * 32 * ITEMS + 32 * i + lane];
+      key[i] = kv.x;
+      vr[i] = kv.y;
+    }
+    cluster_barrier();  // counts published; every CTA's elements are in registers again
     uint32_t below = 0, all = 0;
     if (tid < 256) {
 #pragma unroll
@@ -275,19 +300,18 @@ __global__ void __launch_bounds__(CL_THREADS, 1)
       }
     }
     const uint32_t first = scan256(all, ws);
-    if (tid < 256) off[tid] = first + below;
+    // slot e of a digit's run goes to position off[digit] + e (modulo 2^32)
+    if (tid < 256) off[tid] = first + below - start;
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
       if (!((valid >> i) & 1u)) continue;
-      const uint32_t digit = (key[i] >> shift) & 0xFFu;
-      const uint32_t pos = off[digit] + wc[digit] + (vr[i] >> 17);
-      const uint32_t val = vr[i] & 0x1FFFFu;
+      const uint32_t pos = off[(key[i] >> shift) & 0xFFu] + (uint32_t)(warp * 32 * ITEMS + 32 * i + lane);
       if (last) {
-        perm[pos] = (int)val;
+        perm[pos] = (int)vr[i];
       } else {
         const uint32_t a = map_shared(&sbuf[pos % E], pos / E);
-        asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(key[i]), "r"(val) : "memory");
+        asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(key[i]), "r"(vr[i]) : "memory");
       }
     }
     cluster_barrier();  // scatter complete (and no CTA leaves while others read its counts)
@@ -590,7 +614,7 @@ cudaError_t scatter_orig(const float* in, int64_t Npad, int64_t N, int m, const 
 }
 
 cudaError_t prepare_points(Ctx& c, const float* X, int64_t N, int d, float sigma,
-                           const char* tag, PointsDev& P, cudaStream_t st, bool hilbert) {
+                           const char* tag, PointsDev& P, cudaStream_t st) {
   const std::string t(tag);
   const int d_in = d;
   d = padded_dim(d_in);
@@ -635,7 +659,7 @@ cudaError_t prepare_points(Ctx& c, const float* X, int64_t N, int d, float sigma
   const unsigned kblocks = blocks_for(N, 256);
   switch (dk) {
 #define KRR_KEY(DK, CASE) \
-  CASE: key_kernel<DK><<<kblocks, 256, 0, st>>>(X, N, d_in, dk, bits, hilbert, (const float*)bbp, nbb, (uint32_t*)ka, (int*)va); break;
+  CASE: key_kernel<DK><<<kblocks, 256, 0, st>>>(X, N, d_in, dk, bits, !c.morton, (const float*)bbp, nbb, (uint32_t*)ka, (int*)va); break;
     KRR_KEY(1, case 1) KRR_KEY(2, case 2) KRR_KEY(3, case 3) KRR_KEY(4, case 4)
     KRR_KEY(5, case 5) KRR_KEY(6, case 6) KRR_KEY(7, case 7) KRR_KEY(8, case 8)
     KRR_KEY(0, default)
