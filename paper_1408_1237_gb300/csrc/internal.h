@@ -281,7 +281,29 @@ cudaError_t mvp_acc_launch(Ctx& c, const PointsDev& P, const float* qh, const fl
                            double* dot, cudaStream_t st, const AccCols& cols = AccCols{});
 
 // ---- mvp.cu
+// The partial sums a product leaves for its last kernel.  Row i (sorted) of
+// column c: y = fac[i] * sum_sp part[sp * part_stride + c * Npad + i] + shift *
+// qdiag[c * Npad + i], with part2 / splits2 in place of part / splits where
+// the row's super-block is direct-form (sb_flag 0; sb_flag null: part
+// everywhere).
+struct ProdSums {
+  const double* part;
+  int splits;
+  const double* part2;
+  int splits2;
+  const int* sb_flag;
+  int64_t part_stride;
+  int64_t N, Npad;
+  const float* fac;
+  const float* qdiag;
+  float shift;
+};
+
 struct MvpOut {
+  // if set, called instead of launching the finalize kernel (the fields below
+  // but `active` are then ignored): a solver's own kernel consumes the sums
+  cudaError_t (*finish)(void* arg, const ProdSums& sums, cudaStream_t st) = nullptr;
+  void* finish_arg = nullptr;
   // y = alpha * (K_hat q + shift q) + beta * u, sorted order
   float alpha = 1.f, beta = 0.f;
   const float* u = nullptr;

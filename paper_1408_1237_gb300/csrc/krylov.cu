@@ -105,17 +105,16 @@ __device__ __forceinline__ int col_flag(const KState* S, int pred) {
   }
 }
 
-// One arrival per column, by one thread, once the column's flag `pred` is
-// final.  The last column to arrive publishes whether any column's flag is
-// set (in G and, when cc is in use, as the loop condition).
-__device__ void group_arrive(const KState* S0, int ncols, Group* G, int pred, Cond cc) {
-  __threadfence();
-  if (atomicAdd(&G->ticket, 1u) != (unsigned)(ncols - 1)) return;
-  __threadfence();
-  int any = 0;
-  for (int c = 0; c < ncols; ++c) any |= col_flag(S0 + c, pred);
-  if (pred == PRED_CG) G->cg_any = any;
-  else G->arn_any = any;
+// One arrival per column, by one thread, with whether the column's CG goes on.
+// The last column to arrive publishes whether any does (in G and, when cc is
+// in use, as the loop condition).  Count and flags travel in one atomic
+// (count in the low half, continuing columns in the high half), so nothing is
+// read back from the columns and no fence is needed.
+__device__ __forceinline__ void group_arrive(Group* G, int ncols, int goes_on, Cond cc) {
+  const unsigned seen = atomicAdd(&G->ticket, 1u + ((unsigned)goes_on << 16));
+  if ((seen & 0xFFFFu) != (unsigned)(ncols - 1)) return;
+  const int any = (seen >> 16) + goes_on > 0;
+  G->cg_any = any;
   G->ticket = 0u;
   set_cond(cc, any);
 }
@@ -168,7 +167,7 @@ __global__ void cg_init_kernel(KState* S0, const double* __restrict__ V, int64_t
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       S->cg_cont = 0;
       S->stepping = 0;
-      group_arrive(S0, gridDim.y, G, PRED_CG, cc);
+      group_arrive(G, gridDim.y, 0, cc);
     }
     return;
   }
@@ -190,7 +189,7 @@ __global__ void cg_init_kernel(KState* S0, const double* __restrict__ V, int64_t
     S->cg_brk = 0;
     S->cg_cont = (!identity && tot > 0.0) ? 1 : 0;
     S->stepping = 1;
-    group_arrive(S0, gridDim.y, G, PRED_CG, cc);
+    group_arrive(G, gridDim.y, S->cg_cont, cc);
   }
 }
 
@@ -201,7 +200,7 @@ __global__ void cg_update_kernel(KState* S0, float* __restrict__ z, float* __res
   __shared__ double red[8];
   KRR_COL;
   if (!S->cg_cont) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) group_arrive(S0, gridDim.y, G, PRED_CG, cc);
+    if (blockIdx.x == 0 && threadIdx.x == 0) group_arrive(G, gridDim.y, 0, cc);
     return;
   }
   const float a = (float)S->alpha;
@@ -221,7 +220,7 @@ __global__ void cg_update_kernel(KState* S0, float* __restrict__ z, float* __res
     if (S->cg_brk) S->breakdowns += 1;
     const bool more = !S->cg_brk && S->k < S->maxit && tot > S->eps2 * S->rho0 && isfinite(tot);
     S->cg_cont = more ? 1 : 0;
-    group_arrive(S0, gridDim.y, G, PRED_CG, cc);
+    group_arrive(G, gridDim.y, more, cc);
   }
 }
 
@@ -232,6 +231,150 @@ __global__ void cg_p_kernel(KState* S0, const float* __restrict__ r, float* __re
   if (!S->cg_cont) return;
   const float b = (float)S->beta;
   KRR_GRID_LOOP(i) p[co + i] = fmaf(b, p[co + i], r[co + i]);
+}
+
+// ---- a whole CG step after the product's partial sums, in one launch for Np <=
+// STEP_MAX_NP: M p from the sums, alpha = rho / p.Mp, z += alpha p, r -= alpha
+// M p, rho' = |r|^2, beta = rho'/rho, the continuation test and p = r + beta p.
+// One cluster of STEP_CL CTAs per column: a thread keeps its R rows in
+// registers from the first phase to the last (M p is never written), and the
+// two dot products are exchanged through distributed shared memory, so the
+// step needs two cluster barriers instead of the finalize, update and p
+// kernels with their two ticket reductions through global memory (7.1, 7.9
+// and 1.7 us at 2,000 points; 20.9, 15.4 and 3.4 us with 16 columns).
+// What remains is latency, most of it of the FP64 pipe (2 operations per clock
+// and SM): the column is spread over 8 SMs, sums are trees (256 values in one
+// warp: 12 warp additions, 8 deep), the state is read while the sums load, and
+// 1 / rho is formed meanwhile, which leaves one division on the path.
+constexpr int STEP_CL = 8;
+constexpr int STEP_T = 256;
+// above, 8 SMs per column take longer over the FP64 sums than the three
+// kernels on all SMs (16384 rows: about 4 us of FP64 at 8 splits)
+constexpr int64_t STEP_MAX_NP = 16384;
+constexpr int CG_UNROLL = 4;  // CG steps per turn of the graph's loop
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+__device__ __forceinline__ double tree8(const double* u) {
+  return ((u[0] + u[1]) + (u[2] + u[3])) + ((u[4] + u[5]) + (u[6] + u[7]));
+}
+
+// Cluster-wide sum of v (fixed order: threads, then CTAs); every thread of
+// every CTA gets it.  slot: STEP_CL doubles, used once per launch.  The first
+// call follows a cluster_arrive() and waits for it (every CTA has started).
+template <bool FIRST>
+__device__ __forceinline__ double cluster_sum(double v, double* buf, double* slot, int rank) {
+  const int t = threadIdx.x;
+  buf[t] = v;
+  __syncthreads();
+  double s = 0.0;
+  if (t < 32) {
+    double u[STEP_T / 32];
+#pragma unroll
+    for (int k = 0; k < STEP_T / 32; ++k) u[k] = buf[32 * k + t];
+    s = warp_sum(tree8(u));
+  }
+  if (FIRST) cluster_wait();
+  if (t < STEP_CL) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(slot + rank)), "r"(t));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(s) : "memory");
+  }
+  cluster_arrive();
+  cluster_wait();
+  return tree8(slot);
+}
+
+template <int R>
+__global__ void __launch_bounds__(STEP_T)
+    cg_step_kernel(KState* S0, const ProdSums f, float* __restrict__ z, float* __restrict__ r,
+                   float* __restrict__ p, Group* G, Cond cc) {
+  static_assert(STEP_CL == 8 && STEP_T == 256 && SB == STEP_T, "tree8 and the block of a super-block flag");
+  __shared__ double buf[STEP_T], slot[2][STEP_CL];
+  __shared__ float coef;
+  const int t = threadIdx.x, rank = blockIdx.x, col = blockIdx.y;
+  KState* S = S0 + col;
+  // the state, the vectors and the sums all load at once; only rank 0's last
+  // thread action changes the state, after every CTA has read it
+  const int cont = S->cg_cont, k0 = S->k, maxit = S->maxit, brk0 = S->cg_brk;
+  const double rho = S->rho, stop = S->eps2 * S->rho0;
+  const int64_t co = (int64_t)col * f.Npad;
+  float pv[R], rv[R], zv[R], mp[R], fc[R];
+  double sum[R];
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    const int64_t i0 = (int64_t)(k * STEP_CL + rank) * STEP_T, i = i0 + t;
+    pv[k] = rv[k] = zv[k] = mp[k] = fc[k] = 0.f;
+    sum[k] = 0.0;
+    if (i >= f.Npad) continue;
+    pv[k] = p[co + i];
+    rv[k] = r[co + i];
+    zv[k] = z[co + i];
+    if (i >= f.N) continue;
+    fc[k] = f.fac[i];
+    const bool second = f.sb_flag && f.sb_flag[i0 / SB] == 0;
+    const double* part = (second ? f.part2 : f.part) + co + i;
+    const int splits = second ? f.splits2 : f.splits;
+#pragma unroll 8
+    for (int sp = 0; sp < splits; ++sp) sum[k] += part[(int64_t)sp * f.part_stride];  // as the finalize kernel
+  }
+  if (!cont) {  // uniform over the cluster
+    if (rank == 0 && t == 0) group_arrive(G, gridDim.y, 0, cc);
+    return;
+  }
+  cluster_arrive();
+  double acc = 0.0;
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    // the finalize kernel's roundings
+    const double y = fma((double)f.shift, (double)pv[k], __dmul_rn((double)fc[k], sum[k]));
+    mp[k] = (float)y;
+    acc += y * (double)pv[k];
+  }
+  const double inv_rho = t == 0 && rho > 0.0 ? 1.0 / rho : 0.0;
+  const double pAp = cluster_sum<true>(acc, buf, slot[0], rank);
+  const bool good = pAp > 0.0 && isfinite(pAp);
+  double alpha = 0.0;
+  if (t == 0) {
+    alpha = good ? rho / pAp : 0.0;
+    coef = (float)alpha;
+  }
+  __syncthreads();
+  const float a = coef;
+  acc = 0.0;
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    zv[k] = fmaf(a, pv[k], zv[k]);
+    rv[k] = fmaf(-a, mp[k], rv[k]);
+    acc += (double)rv[k] * (double)rv[k];
+  }
+  const double rr = cluster_sum<false>(acc, buf, slot[1], rank);
+  const bool brk = brk0 || !good;
+  const bool more = !brk && k0 + 1 < maxit && rr > stop && isfinite(rr);
+  if (t == 0) coef = (float)(rr * inv_rho);
+  __syncthreads();
+  const float b = coef;
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    const int64_t i = (int64_t)(k * STEP_CL + rank) * STEP_T + t;
+    if (i >= f.Npad) continue;
+    z[co + i] = zv[k];
+    r[co + i] = rv[k];
+    if (more) p[co + i] = fmaf(b, pv[k], rv[k]);
+  }
+  if (rank == 0 && t == 0) {
+    S->pAp = pAp;
+    S->alpha = alpha;
+    S->beta = rr * inv_rho;
+    S->rho = rr;
+    S->k = k0 + 1;
+    S->inner_total += 1;
+    if (!good) S->cg_brk = 1;
+    if (brk) S->breakdowns += 1;
+    S->cg_cont = more;
+    group_arrive(G, gridDim.y, more, cc);
+  }
 }
 
 // ------------------------------------------------------------- Arnoldi ---
@@ -829,10 +972,39 @@ struct Solver {
     return e;
   }
 
+  // The rest of a CG step from the product's partial sums (MvpOut::finish)
+  static cudaError_t cg_step(void* arg, const ProdSums& sums, cudaStream_t st) {
+    Solver& s = *(Solver*)arg;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(STEP_CL, (unsigned)s.mc);
+    cfg.blockDim = dim3(STEP_T);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = STEP_CL;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const int64_t rows = (s.Np + STEP_CL * STEP_T - 1) / (STEP_CL * STEP_T);  // per thread
+    auto* kernel = rows <= 1 ? cg_step_kernel<1> : rows <= 2 ? cg_step_kernel<2>
+                   : rows <= 4 ? cg_step_kernel<4> : cg_step_kernel<8>;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, s.S, sums, s.z, s.rr, s.p, s.G, s.cg_c);
+    count_launch();
+    return e;
+  }
+
   // ---- one CG iteration on the inner operator M p = K_hat p + mshift p,
   // for every column whose CG continues
   cudaError_t cg_iteration() {
     MvpOut o;
+    if (Np <= STEP_MAX_NP) {
+      o.active = &G->cg_any;
+      o.finish = cg_step;
+      o.finish_arg = this;
+      return mc == 1 ? mvp_launch(c, P, P, p, p, mshift, inner_prec, o, st)
+                     : mvp_multi_launch(c, P, P, p, mc, p, mshift, inner_prec, o, st);
+    }
     o.out_f = Mp;
     o.dotw = p;
     o.dot = &S->pAp;
@@ -1009,7 +1181,16 @@ cudaError_t fill_restart_body(Solver& s, cudaGraph_t rbody, double tol_stop) {
        })))
     return e;
   if ((e = add_while(abody, s.cg_c.h, &cbody))) return e;
-  if ((e = capture_into(s.st, cbody, [&]() -> cudaError_t { return s.cg_iteration(); }))) return e;
+  // several predicated CG steps per turn of the loop: a step of a small problem
+  // costs less than the loop's own turn (a step after the last column has
+  // stopped only reads its flag)
+  const int unroll = s.Np <= STEP_MAX_NP ? CG_UNROLL : 1;
+  if ((e = capture_into(s.st, cbody, [&]() -> cudaError_t {
+         cudaError_t ee = cudaSuccess;
+         for (int k = 0; k < unroll && !ee; ++k) ee = s.cg_iteration();
+         return ee;
+       })))
+    return e;
   if ((e = capture_into(s.st, abody, [&]() -> cudaError_t { return s.arnoldi_tail(); }))) return e;
   return capture_into(s.st, rbody, [&]() -> cudaError_t { return s.cycle_tail(tol_stop); });
 }

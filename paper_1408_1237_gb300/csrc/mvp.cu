@@ -479,19 +479,7 @@ __global__ void __launch_bounds__(NT, (D > 8 ? 1 : 2)) mvp_dirm_kernel(const Mvp
   }
 }
 
-struct FinParams {
-  const double* part;
-  int splits;
-  // multi-column products: targets of direct-form super-blocks (sb_flag 0)
-  // take their sums from part2 (splits2 splits) instead
-  const double* part2;
-  int splits2;
-  const int* sb_flag;
-  int64_t part_stride;
-  int64_t N, Npad;
-  const float* fac;
-  const float* qdiag;
-  float shift;
+struct FinParams : ProdSums {
   MvpOut o;
   double* dot_part;        // [columns][gridDim.x] per-block dot partials
   unsigned int* dot_count; // [columns] arrival counters (reset by the last block)
@@ -1126,6 +1114,7 @@ cudaError_t tcx_path(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, const flo
   f.dot_count = (unsigned*)dcnt;
   f.row_lo = c.row_lo;
   f.row_hi = c.row_hi;
+  if (o.finish) return o.finish(o.finish_arg, f, st);
   mvp_finalize_kernel<<<fin_blocks, 256, 0, st>>>(f); count_launch();
   return cudaGetLastError();
 }
@@ -1208,6 +1197,7 @@ cudaError_t mvp_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, const f
   f.dot_count = (unsigned*)dcnt;
   f.row_lo = c.row_lo;
   f.row_hi = c.row_hi;
+  if (o.finish) return o.finish(o.finish_arg, f, st);
   mvp_finalize_kernel<<<fin_blocks, 256, 0, st>>>(f); count_launch();
   return cudaGetLastError();
 }
@@ -1343,6 +1333,7 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, c
   f.dot_count = (unsigned*)dcnt;
   f.row_lo = c.row_lo;
   f.row_hi = c.row_hi;
+  if (o.finish) return o.finish(o.finish_arg, f, st);
   mvp_finalize_kernel<<<dim3(fin_blocks, (unsigned)m), 256, 0, st>>>(f); count_launch();
   return cudaGetLastError();
 }
