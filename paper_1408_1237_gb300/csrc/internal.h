@@ -304,6 +304,9 @@ struct MvpOut {
   // but `active` are then ignored): a solver's own kernel consumes the sums
   cudaError_t (*finish)(void* arg, const ProdSums& sums, cudaStream_t st) = nullptr;
   void* finish_arg = nullptr;
+  // an inner product of a solver's preconditioner, which tolerates rounding:
+  // several columns take the tensor-core kernels' less exact form
+  bool inner = false;
   // y = alpha * (K_hat q + shift q) + beta * u, sorted order
   float alpha = 1.f, beta = 0.f;
   const float* u = nullptr;
@@ -347,9 +350,11 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& T, const PointsDev& S, con
                              const float* qdiag, float shift, krr_precision prec, const MvpOut& o,
                              cudaStream_t st);
 // ---- mvp_tc.cu: tensor-core partial sums of the expanded-form warp blocks
+// fine = false: the form for the inner products of a solver's preconditioner
+// (KRR_FP32 only; see the kernel).
 // dry = true only sets the kernel attributes (before any graph capture).
 cudaError_t mvp_tc_partials(Ctx& c, const PointsDev& T, const PointsDev& S, const float* Q, int m,
-                            bool split, bool bf, int splits, int tiles_per_split, double* part,
+                            krr_precision prec, bool fine, int splits, int tiles_per_split, double* part,
                             float* fac, const int* active, cudaStream_t st, bool dry = false);
 // ---- mvp_tc.cu: single-column float32-grade partial sums of the
 // expanded-form super-blocks (exponent on the tensor cores, EX2 + FMA per
@@ -370,7 +375,10 @@ cudaError_t mvp_umma_partials(Ctx& c, const PointsDev& T, const PointsDev& S, co
 cudaError_t mvp_dirtc_partials(Ctx& c, const PointsDev& T, const PointsDev& S, const float* Q, int m,
                                krr_precision prec, int splits, int tiles_per_split, int64_t slot0,
                                const int* tn_exp, double* part, float* fac, const int* active,
-                               cudaStream_t st, bool dry = false);
+                               bool fine, cudaStream_t st, bool dry = false);
+// Whether m columns of a product over the targets T cost less in one pass
+// (mvp_multi_launch) than as m single-column products.
+bool multi_pays(const Ctx& c, const PointsDev& T, int m, krr_precision prec);
 // Workspace and attributes of mvp_multi_launch with m columns and prec.
 cudaError_t mvp_multi_reserve(Ctx& c, const PointsDev& T, const PointsDev& S, int m,
                               krr_precision prec, cudaStream_t st);

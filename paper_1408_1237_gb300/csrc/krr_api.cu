@@ -640,12 +640,20 @@ krr_status krr_kernel_mvp_rect(krr_handle h, const float* Xt, int64_t Nt, const 
     void* qs;
     if ((e = c.ws.get("mvp.qs", sizeof(float) * S.Npad * m, &qs))) return cuda_error(c, e, fn);
     if ((e = gather_sorted(dQ, Ns, m, S.perm, S.Npad, (float*)qs, st))) return cuda_error(c, e, fn);
-    for (int col = 0; col < m; ++col) {
+    // columns in as few passes as possible where one pass evaluates each
+    // kernel value for all of its columns at less than their single cost
+    const bool shared = multi_pays(c, T, m, prec);
+    const int passes = shared ? (m + MAX_COLS - 1) / MAX_COLS : m;
+    const int width = (m + passes - 1) / passes;
+    for (int col = 0; col < m; col += width) {
+      const int mc = std::min(width, m - col);
+      const float* qc = (const float*)qs + (size_t)col * S.Npad;
       MvpOut o;
       o.perm = T.perm;
       o.out_orig = dY + (size_t)col * Nt;
-      if ((e = mvp_launch(c, T, S, (const float*)qs + (size_t)col * S.Npad, nullptr, 0.f, prec, o, st)))
-        return cuda_error(c, e, fn);
+      e = mc == 1 ? mvp_launch(c, T, S, qc, nullptr, 0.f, prec, o, st)
+                  : mvp_multi_launch(c, T, S, qc, mc, nullptr, 0.f, prec, o, st);
+      if (e) return cuda_error(c, e, fn);
     }
   }
   if (s4 && (e = cudaMemcpyAsync(Y, dY, sizeof(float) * Nt * m, cudaMemcpyDeviceToHost, st)))

@@ -864,6 +864,7 @@ cudaError_t autotune_mvp(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, int m
   }
   MvpOut o;
   o.out_f = (float*)yv;
+  o.inner = tcgen05_only;  // a solver's choice
   const bool single = m == 1 && prec == KRR_FP32;
   auto run = [&]() {
     return single ? mvp_launch(c, Tp, Sp, (const float*)qv, nullptr, 0.f, prec, o, st)
@@ -1229,9 +1230,10 @@ cudaError_t mvp_multi_reserve(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, 
   MvpParams p{};
   p.nblk = Tp.nsb;
   if (use_dirtc(c, Tp)) {
-    if ((e = mvp_dirtc_partials(c, Tp, Sp, nullptr, m, prec, pd.splits, pd.tiles_per_split, multi_nexp(Tp),
-                                nullptr, nullptr, nullptr, nullptr, st, true)))
-      return e;
+    for (bool fine : {false, true})
+      if ((e = mvp_dirtc_partials(c, Tp, Sp, nullptr, m, prec, pd.splits, pd.tiles_per_split, multi_nexp(Tp),
+                                  nullptr, nullptr, nullptr, nullptr, fine, st, true)))
+        return e;
   } else if ((e = dirm_dispatch(p, Tp.d, Tp.kfam, nullptr, 0, m, SB / 32, multi_nexp(Tp), pd, st, false))) {
     return e;
   }
@@ -1239,8 +1241,24 @@ cudaError_t mvp_multi_reserve(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, 
   if (tc5_on(c, prec, m, Tp))
     return mvp_umma_partials(c, Tp, Sp, nullptr, m, prec == KRR_FP32, prec == KRR_BF16, pt.splits,
                              pt.tiles_per_split, nullptr, nullptr, nullptr, st, true);
-  return mvp_tc_partials(c, Tp, Sp, nullptr, m, prec == KRR_FP32, prec == KRR_BF16, pt.splits,
-                         pt.tiles_per_split, nullptr, nullptr, nullptr, st, true);
+  for (bool fine : {false, true})
+    if ((e = mvp_tc_partials(c, Tp, Sp, nullptr, m, prec, fine, pt.splits, pt.tiles_per_split, nullptr, nullptr,
+                             nullptr, st, true)))
+      return e;
+  return cudaSuccess;
+}
+
+// One column against a pass of 2 to 8, 16 columns on GB300: 131,072 points,
+// d = 3, 2.51 ms against 4.9 to 5.3, 5.8; 20,000 points 148 us against 310 to
+// 322, 440; d = 8, 16,384 points 158 against 339 to 352, 479.  So two columns
+// tie and three gain 1.4 times in one pass.  Above 8 dimensions the pass takes
+// the direct form, where a single column has the tensor cores on compact
+// blocks: d = 16, 16,384 points 134 us against 422 up to 4 columns, 488 up to
+// 8, 749 at 16.
+bool multi_pays(const Ctx& c, const PointsDev& Tp, int m, krr_precision prec) {
+  if (prec != KRR_FP32) return m >= 2;
+  if (Tp.d <= 8) return m >= 3;
+  return m >= (use_tcx(c, Tp) ? 4 : 2);
 }
 
 cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, const float* Q, int m,
@@ -1293,8 +1311,8 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, c
     e = tc5_on(c, prec, m, Tp)
             ? mvp_umma_partials(c, Tp, Sp, Q, m, prec == KRR_FP32, prec == KRR_BF16, pt.splits,
                                 pt.tiles_per_split, (double*)part, p.fac, o.active, st)
-            : mvp_tc_partials(c, Tp, Sp, Q, m, prec == KRR_FP32, prec == KRR_BF16, pt.splits,
-                              pt.tiles_per_split, (double*)part, p.fac, o.active, st);
+            : mvp_tc_partials(c, Tp, Sp, Q, m, prec, !o.inner, pt.splits, pt.tiles_per_split, (double*)part,
+                              p.fac, o.active, st);
     if (e) return e;
   }
   // direct-form super-blocks: all columns in one launch (the weighted sum
@@ -1309,7 +1327,7 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, c
     }
     if (use_dirtc(c, Tp)) {
       if ((e = mvp_dirtc_partials(c, Tp, Sp, Q, m, prec, pd.splits, pd.tiles_per_split, nexp, p.tn_exp,
-                                  (double*)partd, p.fac, o.active, st, false)))
+                                  (double*)partd, p.fac, o.active, !o.inner, st, false)))
         return e;
     } else if ((e = dirm_dispatch(p, Tp.d, Tp.kfam, Q, Sp.Npad, m, SB / 32, nexp, pd, st, true))) {
       return e;

@@ -13,12 +13,21 @@
 // becomes a dense contraction on the tensor cores (mma.sync, 8 columns per
 // MMA), each thread computing the kernel values of the A fragment it owns:
 //   * float32-grade products use tf32 operands split into hi + lo, with
-//     P = Ph + Pl, Ph = P with its low 13 mantissa bits cleared (one logical
-//     operation) and Pl = P - Ph exact (one subtraction): Ph Qh + Pl Qh +
-//     Ph Ql (m16n8k8), relative error per term below 3 * 2^-20.  No format
-//     conversion is needed (tf32 is float32's layout), and tf32 has float32's
-//     exponent range, so small kernel values and large weights keep their
-//     precision;
+//     P = Ph + Pl, Ph of tf32's 11 significant bits and Pl = P - Ph exact (one
+//     subtraction): Ph Qh + Pl Qh + Ph Ql (m16n8k8), relative error per term
+//     below 3 * 2^-20.  No format conversion is needed (tf32 is float32's
+//     layout), and tf32 has float32's exponent range, so small kernel values
+//     and large weights keep their precision.  Two forms (SPLIT):
+//      1: Ph = P with its low bits cleared, one accumulator for all three.  For
+//         the inner products of the solvers' preconditioner.  Relative error
+//         of a product 1.8e-6 (20,011 points, d = 3) to 2.5e-6 (16,385, d = 8);
+//      2: for every other product.  Ph is rounded, which gives the low parts
+//         both signs, so that what the split drops does not add up; the tensor
+//         cores truncate when they accumulate, so Ph Qh goes into fresh
+//         accumulators every FOLD sources, folded in float32, and the two small
+//         products into accumulators of their own.  Error 1.9e-7 and 2.9e-7 in
+//         the same cases, as the single-column float32 kernels (2.4e-7,
+//         3.9e-7), for about 2% more time;
 //   * reduced-precision products (the inner M p of Sec. 5.1) issue P Q with
 //     single f16 or bf16 operands (m16n8k16); f16 kernel values are formed as
 //     2^15 P (the offset enters the exponent) so that small values stay out
@@ -51,6 +60,8 @@ constexpr int DT_RS = 2;                   // raw stages
 constexpr int QS = 264;                    // halves per f16 weight row of a work buffer (256 + pad)
 constexpr int QSW = 260;                   // words per tf32 weight row (256 + pad: conflict-free)
 constexpr uint32_t TF32_MASK = 0xFFFFE000u;  // clears the 13 mantissa bits tf32 drops
+constexpr uint32_t TF32_HALF = 0x1000u;      // half a unit of tf32's last place
+constexpr int FOLD = 64;                     // sources per accumulation of Ph Qh
 constexpr float F16_OFFSET = 15.f;         // f16 kernel values are 2^15 P
 constexpr float kLog2eDt = 1.4426950408889634f;
 
@@ -124,6 +135,13 @@ __device__ __forceinline__ void mma_1688_tf32(float (&d)[4], const uint32_t (&a)
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// v rounded to tf32, half away from zero.  (The largest finite weights keep
+// their value: rounding up would carry into infinity.)
+__device__ __forceinline__ uint32_t tf32_hi(float v) {
+  const uint32_t u = __float_as_uint(v), up = u + TF32_HALF;
+  return ((up & 0x7F800000u) == 0x7F800000u ? u : up) & TF32_MASK;
+}
+
 // Kernel values of two pairs from their squared raw distances, times 2^off.
 template <int KF>
 __device__ __forceinline__ float2 pair_values(float2 r2, float s, float off) {
@@ -144,23 +162,23 @@ __device__ __forceinline__ float2 pair_values(float2 r2, float s, float off) {
   }
 }
 
-template <int D, int NRT, bool SPLIT>
+template <int D, int NRT, int SPLIT>
 constexpr uint32_t dt_raw_floats() {
   return (uint32_t)(D + 8 * NRT) * TS;
 }
 // work buffer: D x 256 permuted negated coordinates, then the weight rows of
 // 8 NRT columns: tf32 hi and lo at QSW words each (split), else QS halves
-template <int D, int NRT, bool SPLIT>
+template <int D, int NRT, int SPLIT>
 constexpr uint32_t dt_work_bytes() {
   return (uint32_t)(sizeof(float) * D * TS +
                     (SPLIT ? 4 * 2 * 8 * NRT * QSW : 2 * 8 * NRT * QS));
 }
-template <int D, int NRT, bool SPLIT>
+template <int D, int NRT, int SPLIT>
 constexpr size_t dt_smem_bytes() {
   return sizeof(float) * DT_RS * dt_raw_floats<D, NRT, SPLIT>() + 2 * (size_t)dt_work_bytes<D, NRT, SPLIT>();
 }
 
-template <int D, int NRT, bool SPLIT, bool BF, int KF>
+template <int D, int NRT, int SPLIT, bool BF, int KF>
 __global__ void __launch_bounds__(DT_THREADS, 1) mvp_dirtc_kernel(const DtParams p) {
   using H = HalfOps<BF>;
   constexpr int MC = 8 * NRT;
@@ -197,11 +215,13 @@ __global__ void __launch_bounds__(DT_THREADS, 1) mvp_dirtc_kernel(const DtParams
   const int t_begin = blockIdx.y * p.tiles_per_split;
   const int nt = min(p.ntiles, t_begin + p.tiles_per_split) - t_begin;
 
-  float acc[NRT][4], S[NRT][4], C[NRT][4];
+  // acc: P Q of the tile (SPLIT 2: Ph Qh of the current FOLD sources);
+  // low: SPLIT 2, Pl Qh + Ph Ql of the tile
+  float acc[NRT][4], low[NRT][4], S[NRT][4], C[NRT][4];
 #pragma unroll
   for (int rt = 0; rt < NRT; ++rt)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) acc[rt][e] = S[rt][e] = C[rt][e] = 0.f;
+    for (int e = 0; e < 4; ++e) acc[rt][e] = low[rt][e] = S[rt][e] = C[rt][e] = 0.f;
 
   auto issue = [&](int r) {
     const int stage = r % DT_RS;
@@ -234,7 +254,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) mvp_dirtc_kernel(const DtParams
       for (int e = tid; e < MC * TS; e += DT_THREADS) {
         const int c = e / TS, j = e % TS;
         const float v = c < p.m ? rs[(D + c) * TS + j] : 0.f;
-        const uint32_t hi = __float_as_uint(v) & TF32_MASK;
+        const uint32_t hi = SPLIT == 2 ? tf32_hi(v) : __float_as_uint(v) & TF32_MASK;
         qw[c * QSW + j] = hi;
         qw[(MC + c) * QSW + j] = __float_as_uint(v - __uint_as_float(hi));
       }
@@ -317,7 +337,8 @@ __global__ void __launch_bounds__(DT_THREADS, 1) mvp_dirtc_kernel(const DtParams
         for (int hf = 0; hf < 2; ++hf)
 #pragma unroll
           for (int w = 0; w < 4; ++w) {
-            ah[hf][w] = __float_as_uint(vv[hf][w]) & TF32_MASK;
+            // P <= 1: rounding up does not overflow
+            ah[hf][w] = (__float_as_uint(vv[hf][w]) + (SPLIT == 2 ? TF32_HALF : 0u)) & TF32_MASK;
             al[hf][w] = __float_as_uint(vv[hf][w] - __uint_as_float(ah[hf][w]));
           }
 #pragma unroll
@@ -329,8 +350,8 @@ __global__ void __launch_bounds__(DT_THREADS, 1) mvp_dirtc_kernel(const DtParams
             const uint32_t b0 = qw[c * QSW + j0], b1 = qw[c * QSW + j0 + 4];
             const uint32_t l0 = qw[(MC + c) * QSW + j0], l1 = qw[(MC + c) * QSW + j0 + 4];
             mma_1688_tf32(acc[rt], ah[hf], b0, b1);
-            mma_1688_tf32(acc[rt], al[hf], b0, b1);
-            mma_1688_tf32(acc[rt], ah[hf], l0, l1);
+            mma_1688_tf32(SPLIT == 2 ? low[rt] : acc[rt], al[hf], b0, b1);
+            mma_1688_tf32(SPLIT == 2 ? low[rt] : acc[rt], ah[hf], l0, l1);
           }
         }
       } else {
@@ -348,6 +369,15 @@ __global__ void __launch_bounds__(DT_THREADS, 1) mvp_dirtc_kernel(const DtParams
           mma_16816<BF>(acc[rt], ph, b0, b1);
         }
       }
+      if (SPLIT == 2 && (kk & (FOLD / 16 - 1)) == FOLD / 16 - 1 && kk != TS / 16 - 1) {
+#pragma unroll
+        for (int rt = 0; rt < NRT; ++rt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            kahan_add(S[rt][e], C[rt][e], acc[rt][e]);
+            acc[rt][e] = 0.f;
+          }
+      }
     }
     // f16 sums carry the 2^15 offset of the kernel values
     constexpr float unscale = (SPLIT || BF) ? 1.f : 1.f / 32768.f;
@@ -355,8 +385,8 @@ __global__ void __launch_bounds__(DT_THREADS, 1) mvp_dirtc_kernel(const DtParams
     for (int rt = 0; rt < NRT; ++rt)
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        kahan_add(S[rt][e], C[rt][e], acc[rt][e] * unscale);
-        acc[rt][e] = 0.f;
+        kahan_add(S[rt][e], C[rt][e], SPLIT == 2 ? acc[rt][e] + low[rt][e] : acc[rt][e] * unscale);
+        acc[rt][e] = low[rt][e] = 0.f;
       }
     __syncthreads();
   }
@@ -378,7 +408,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) mvp_dirtc_kernel(const DtParams
     }
 }
 
-template <int D, int NRT, bool SPLIT, bool BF, int KF>
+template <int D, int NRT, int SPLIT, bool BF, int KF>
 cudaError_t dt_launch(const DtParams& p, int64_t nctas, int splits, cudaStream_t st, bool launch) {
   static bool done[128] = {};
   int dev = 0;
@@ -399,33 +429,36 @@ cudaError_t dt_launch(const DtParams& p, int64_t nctas, int splits, cudaStream_t
 
 template <int D, int KF>
 cudaError_t dt_dispatch_d(const DtParams& p, int64_t nctas, int splits, krr_precision prec,
-                          cudaStream_t st, bool launch) {
+                          bool fine, cudaStream_t st, bool launch) {
   const bool two = p.m > 8;
+  if ((KF != 0 || prec == KRR_FP32) && fine)
+    return two ? dt_launch<D, 2, 2, false, KF>(p, nctas, splits, st, launch)
+               : dt_launch<D, 1, 2, false, KF>(p, nctas, splits, st, launch);
   if (KF != 0 || prec == KRR_FP32)
-    return two ? dt_launch<D, 2, true, false, KF>(p, nctas, splits, st, launch)
-               : dt_launch<D, 1, true, false, KF>(p, nctas, splits, st, launch);
+    return two ? dt_launch<D, 2, 1, false, KF>(p, nctas, splits, st, launch)
+               : dt_launch<D, 1, 1, false, KF>(p, nctas, splits, st, launch);
   if constexpr (KF == 0) {
     if (prec == KRR_BF16)
-      return two ? dt_launch<D, 2, false, true, 0>(p, nctas, splits, st, launch)
-                 : dt_launch<D, 1, false, true, 0>(p, nctas, splits, st, launch);
-    return two ? dt_launch<D, 2, false, false, 0>(p, nctas, splits, st, launch)
-               : dt_launch<D, 1, false, false, 0>(p, nctas, splits, st, launch);
+      return two ? dt_launch<D, 2, 0, true, 0>(p, nctas, splits, st, launch)
+                 : dt_launch<D, 1, 0, true, 0>(p, nctas, splits, st, launch);
+    return two ? dt_launch<D, 2, 0, false, 0>(p, nctas, splits, st, launch)
+               : dt_launch<D, 1, 0, false, 0>(p, nctas, splits, st, launch);
   }
   return cudaErrorNotSupported;
 }
 
 template <int KF>
 cudaError_t dt_dispatch(const DtParams& p, int d, int64_t nctas, int splits, krr_precision prec,
-                        cudaStream_t st, bool launch) {
+                        bool fine, cudaStream_t st, bool launch) {
   switch (d) {
-    case 1: return dt_dispatch_d<1, KF>(p, nctas, splits, prec, st, launch);
-    case 2: return dt_dispatch_d<2, KF>(p, nctas, splits, prec, st, launch);
-    case 3: return dt_dispatch_d<3, KF>(p, nctas, splits, prec, st, launch);
-    case 4: return dt_dispatch_d<4, KF>(p, nctas, splits, prec, st, launch);
-    case 5: return dt_dispatch_d<5, KF>(p, nctas, splits, prec, st, launch);
-    case 6: return dt_dispatch_d<6, KF>(p, nctas, splits, prec, st, launch);
-    case 7: return dt_dispatch_d<7, KF>(p, nctas, splits, prec, st, launch);
-    case 8: return dt_dispatch_d<8, KF>(p, nctas, splits, prec, st, launch);
+    case 1: return dt_dispatch_d<1, KF>(p, nctas, splits, prec, fine, st, launch);
+    case 2: return dt_dispatch_d<2, KF>(p, nctas, splits, prec, fine, st, launch);
+    case 3: return dt_dispatch_d<3, KF>(p, nctas, splits, prec, fine, st, launch);
+    case 4: return dt_dispatch_d<4, KF>(p, nctas, splits, prec, fine, st, launch);
+    case 5: return dt_dispatch_d<5, KF>(p, nctas, splits, prec, fine, st, launch);
+    case 6: return dt_dispatch_d<6, KF>(p, nctas, splits, prec, fine, st, launch);
+    case 7: return dt_dispatch_d<7, KF>(p, nctas, splits, prec, fine, st, launch);
+    case 8: return dt_dispatch_d<8, KF>(p, nctas, splits, prec, fine, st, launch);
     default: return cudaErrorNotSupported;
   }
 }
@@ -435,7 +468,7 @@ cudaError_t dt_dispatch(const DtParams& p, int d, int64_t nctas, int splits, krr
 cudaError_t mvp_dirtc_partials(Ctx& c, const PointsDev& T, const PointsDev& S, const float* Q, int m,
                                krr_precision prec, int splits, int tiles_per_split, int64_t slot0,
                                const int* tn_exp, double* part, float* fac, const int* active,
-                               cudaStream_t st, bool dry) {
+                               bool fine, cudaStream_t st, bool dry) {
   if (T.d < 1 || T.d > 8 || m < 1 || m > MAX_COLS) return cudaErrorNotSupported;
   DtParams p{};
   p.xt = T.xs;
@@ -459,9 +492,9 @@ cudaError_t mvp_dirtc_partials(Ctx& c, const PointsDev& T, const PointsDev& S, c
   p.row_lo = c.row_lo;
   p.row_hi = c.row_hi;
   const int64_t nctas = std::max<int64_t>(1, T.nsb - slot0);
-  if (T.kfam == KRR_KERNEL_MATERN32) return dt_dispatch<1>(p, T.d, nctas, splits, prec, st, !dry);
+  if (T.kfam == KRR_KERNEL_MATERN32) return dt_dispatch<1>(p, T.d, nctas, splits, prec, fine, st, !dry);
   if (T.kfam != KRR_KERNEL_GAUSSIAN) return cudaErrorNotSupported;
-  return dt_dispatch<0>(p, T.d, nctas, splits, prec, st, !dry);
+  return dt_dispatch<0>(p, T.d, nctas, splits, prec, fine, st, !dry);
 }
 
 }  // namespace krr

@@ -158,7 +158,13 @@ __device__ __forceinline__ float kv_value(const float (&h)[D + 1], const float (
   return v;
 }
 
-template <int D, int MT, int NRT, bool SPLIT, bool BF>
+// SPLIT: 0 single operands; 1 hi + lo, for the inner products of the solvers'
+// preconditioner; 2 hi + lo with Ph Qh in fresh accumulators every FOLD sources
+// (the tensor cores truncate when they accumulate) and the small products in
+// accumulators of their own, for every other float32 product.  Relative error
+// at 131,072 points in the cube 1.5e-6 with 1 and 2.8e-7 with 2, as the
+// single-column kernels (2.5e-7), for 2 to 5% more time.
+template <int D, int MT, int NRT, int SPLIT, bool BF>
 __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
   using L = ExpLayout<D>;
   using H = Half<BF>;
@@ -222,14 +228,17 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
   const int t_begin = blockIdx.y * p.tiles_per_split;
   const int nt = min(p.ntiles, t_begin + p.tiles_per_split) - t_begin;
 
-  float acc[MT][NRT][4];
+  // acc: P Q of the tile (SPLIT 2: Ph Qh of the current FOLD sources);
+  // low: SPLIT 2, Pl Qh + Ph Ql of the tile
+  constexpr int FOLD = 64;
+  float acc[MT][NRT][4], low[MT][NRT][4];
   float S[MT][NRT][4], C[MT][NRT][4];
 #pragma unroll
   for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
     for (int rt = 0; rt < NRT; ++rt)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) acc[mt][rt][e] = S[mt][rt][e] = C[mt][rt][e] = 0.f;
+      for (int e = 0; e < 4; ++e) acc[mt][rt][e] = low[mt][rt][e] = S[mt][rt][e] = C[mt][rt][e] = 0.f;
 
   auto issue = [&](int r) {
     const int stage = r % RS;
@@ -388,10 +397,21 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
         for (int rt = 0; rt < NRT; ++rt) {
           mma16816<BF>(acc[mt][rt], ph, qfh[rt][0], qfh[rt][1]);
           if (SPLIT) {
-            mma16816<BF>(acc[mt][rt], pl, qfh[rt][0], qfh[rt][1]);
-            mma16816<BF>(acc[mt][rt], ph, qfl[rt][0], qfl[rt][1]);
+            mma16816<BF>(SPLIT == 2 ? low[mt][rt] : acc[mt][rt], pl, qfh[rt][0], qfh[rt][1]);
+            mma16816<BF>(SPLIT == 2 ? low[mt][rt] : acc[mt][rt], ph, qfl[rt][0], qfl[rt][1]);
           }
         }
+      }
+      if (SPLIT == 2 && (kk & (FOLD / 16 - 1)) == FOLD / 16 - 1 && kk != TS / 16 - 1) {
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+          for (int rt = 0; rt < NRT; ++rt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              kahan_add(S[mt][rt][e], C[mt][rt][e], acc[mt][rt][e]);
+              acc[mt][rt][e] = 0.f;
+            }
       }
     }
     // fold the tile's sums into compensated float32 accumulators
@@ -401,8 +421,8 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
       for (int rt = 0; rt < NRT; ++rt)
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          kahan_add(S[mt][rt][e], C[mt][rt][e], acc[mt][rt][e]);
-          acc[mt][rt][e] = 0.f;
+          kahan_add(S[mt][rt][e], C[mt][rt][e], SPLIT == 2 ? acc[mt][rt][e] + low[mt][rt][e] : acc[mt][rt][e]);
+          acc[mt][rt][e] = low[mt][rt][e] = 0.f;
         }
     __syncthreads();
   }
@@ -2188,7 +2208,7 @@ cudaError_t tch_launch_typed(const TcParams& p, int splits, cudaStream_t st, boo
   return cudaGetLastError();
 }
 
-template <int D, int MT, int NRT, bool SPLIT, bool BF>
+template <int D, int MT, int NRT, int SPLIT, bool BF>
 cudaError_t launch(const TcParams& p, int splits, int warps, cudaStream_t st, bool dry) {
   using L = ExpLayout<D>;
   constexpr int MC = 8 * NRT;
@@ -2212,33 +2232,26 @@ cudaError_t launch(const TcParams& p, int splits, int warps, cudaStream_t st, bo
   return cudaGetLastError();
 }
 
-template <int D, bool SPLIT, bool BF>
+template <int D, int SPLIT, bool BF>
 cudaError_t dispatch_m(const TcParams& p, int splits, cudaStream_t st, bool dry) {
   // m-tiles per warp: 4 (2 for two groups of right-hand sides with split
-  // accumulators, keeping registers under 128); never beyond the block
-  const int mt_max = p.WB / 16;
-  if (p.m <= 8) {
-    const int MT = std::min(4, mt_max);
-    const int warps = p.WB / (16 * MT);
-    if (MT == 4) return launch<D, 4, 1, SPLIT, BF>(p, splits, warps, st, dry);
-    return launch<D, 2, 1, SPLIT, BF>(p, splits, warps, st, dry);
-  }
-  const int MT = std::min(2, mt_max);
-  return launch<D, 2, 2, SPLIT, BF>(p, splits, p.WB / (16 * MT), st, dry);
+  // accumulators, keeping registers under 128)
+  if (p.m <= 8) return launch<D, 4, 1, SPLIT, BF>(p, splits, SB / (16 * 4), st, dry);
+  return launch<D, 2, 2, SPLIT, BF>(p, splits, SB / (16 * 2), st, dry);
 }
 
 template <int D>
-cudaError_t dispatch_prec(const TcParams& p, int splits, bool split, bool bf, cudaStream_t st,
+cudaError_t dispatch_prec(const TcParams& p, int splits, krr_precision prec, bool fine, cudaStream_t st,
                           bool dry) {
-  if (split)
-    return bf ? dispatch_m<D, true, true>(p, splits, st, dry) : dispatch_m<D, true, false>(p, splits, st, dry);
-  return bf ? dispatch_m<D, false, true>(p, splits, st, dry) : dispatch_m<D, false, false>(p, splits, st, dry);
+  if (prec == KRR_FP32)
+    return fine ? dispatch_m<D, 2, false>(p, splits, st, dry) : dispatch_m<D, 1, false>(p, splits, st, dry);
+  return prec == KRR_BF16 ? dispatch_m<D, 0, true>(p, splits, st, dry) : dispatch_m<D, 0, false>(p, splits, st, dry);
 }
 
 }  // namespace
 
 cudaError_t mvp_tc_partials(Ctx& c, const PointsDev& T, const PointsDev& S, const float* Q, int m,
-                            bool split, bool bf, int splits, int tiles_per_split, double* part,
+                            krr_precision prec, bool fine, int splits, int tiles_per_split, double* part,
                             float* fac, const int* active, cudaStream_t st, bool dry) {
   if (m < 1 || m > 16) return cudaErrorNotSupported;
   TcParams p{};
@@ -2265,14 +2278,14 @@ cudaError_t mvp_tc_partials(Ctx& c, const PointsDev& T, const PointsDev& S, cons
   p.s = S.scale;
   p.active = active;
   switch (T.d) {
-    case 1: return dispatch_prec<1>(p, splits, split, bf, st, dry);
-    case 2: return dispatch_prec<2>(p, splits, split, bf, st, dry);
-    case 3: return dispatch_prec<3>(p, splits, split, bf, st, dry);
-    case 4: return dispatch_prec<4>(p, splits, split, bf, st, dry);
-    case 5: return dispatch_prec<5>(p, splits, split, bf, st, dry);
-    case 6: return dispatch_prec<6>(p, splits, split, bf, st, dry);
-    case 7: return dispatch_prec<7>(p, splits, split, bf, st, dry);
-    case 8: return dispatch_prec<8>(p, splits, split, bf, st, dry);
+    case 1: return dispatch_prec<1>(p, splits, prec, fine, st, dry);
+    case 2: return dispatch_prec<2>(p, splits, prec, fine, st, dry);
+    case 3: return dispatch_prec<3>(p, splits, prec, fine, st, dry);
+    case 4: return dispatch_prec<4>(p, splits, prec, fine, st, dry);
+    case 5: return dispatch_prec<5>(p, splits, prec, fine, st, dry);
+    case 6: return dispatch_prec<6>(p, splits, prec, fine, st, dry);
+    case 7: return dispatch_prec<7>(p, splits, prec, fine, st, dry);
+    case 8: return dispatch_prec<8>(p, splits, prec, fine, st, dry);
     default: return cudaErrorNotSupported;
   }
 }
