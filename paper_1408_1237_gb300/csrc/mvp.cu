@@ -35,9 +35,9 @@
 //    shift term and the fused epilogue (axpy, dot, scatter).
 //  * Other kernel functions (the Matern kernel of Sec. 6.1) take the direct
 //    form in the multi-column CUDA-core kernel, templated on the pair
-//    function (KF): a = s |x_i - x_j| with s = sqrt(3) / h by one reciprocal
-//    square root and one multiply, then (1 + a) 2^(-a log2(e)) by one
-//    MUFU.EX2 and one FMA.
+//    function (KF): a = s |x_i - x_j| with s = sqrt(3) / h by one square root
+//    on the special-function unit and one multiply, then (1 + a) 2^(-a log2(e))
+//    by one MUFU.EX2 and one FMA.
 #include <algorithm>
 #include <cmath>
 
@@ -137,10 +137,8 @@ __device__ __forceinline__ void compute_expanded(const float* __restrict__ cb,
 constexpr float kLog2e = 1.4426950408889634f;  // log2(e) = 1 / ln 2
 
 // Matern 3/2 value from the squared raw distance: a = s r, (1 + a) 2^(-a log2 e).
-// r = r2 / sqrt(r2) through the reciprocal square root (a 2-ulp routine); the
-// clamp keeps r2 = 0 (a point against itself) at a = 0 instead of 0 * inf.
 __device__ __forceinline__ float matern32_value(float r2, float s) {
-  const float a = s * (r2 * rsqrtf(fmaxf(r2, 1e-30f)));
+  const float a = s * sqrt_mufu(r2);
   const float e = ex2(a * -kLog2e);
   return fmaf(a, e, e);
 }
@@ -181,11 +179,9 @@ __device__ __forceinline__ void compute_direct(const float* __restrict__ cb,
         e1.x = ex2(r1.x);
         e1.y = ex2(r1.y);
       } else {
-        // a = s r (r = r^2 rsqrt(r^2), clamped at r^2 = 0), then (1 + a) 2^(-a log2 e)
-        const float2 a0 = fmul2(sv, fmul2(r0, make_float2(rsqrtf(fmaxf(r0.x, 1e-30f)),
-                                                          rsqrtf(fmaxf(r0.y, 1e-30f)))));
-        const float2 a1 = fmul2(sv, fmul2(r1, make_float2(rsqrtf(fmaxf(r1.x, 1e-30f)),
-                                                          rsqrtf(fmaxf(r1.y, 1e-30f)))));
+        // a = s r, then (1 + a) 2^(-a log2 e)
+        const float2 a0 = fmul2(sv, make_float2(sqrt_mufu(r0.x), sqrt_mufu(r0.y)));
+        const float2 a1 = fmul2(sv, make_float2(sqrt_mufu(r1.x), sqrt_mufu(r1.y)));
         const float2 t0 = fmul2(a0, nl2e), t1 = fmul2(a1, nl2e);
         e0 = make_float2(ex2(t0.x), ex2(t0.y));
         e1 = make_float2(ex2(t1.x), ex2(t1.y));

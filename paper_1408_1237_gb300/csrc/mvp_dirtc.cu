@@ -149,13 +149,12 @@ __device__ __forceinline__ float2 pair_values(float2 r2, float s, float off) {
     const float2 e = ffma2(r2, make_float2(-s * s, -s * s), make_float2(off, off));
     return make_float2(ex2(e.x), ex2(e.y));
   } else {
-    // Matern 3/2: a = s r, (1 + a) 2^(off - a log2 e); r through the
-    // reciprocal square root, the clamp keeping r2 = 0 at a = 0
+    // Matern 3/2: a = s r, (1 + a) 2^(off - a log2 e)
     float2 v;
-    float a = s * (r2.x * rsqrtf(fmaxf(r2.x, 1e-30f)));
+    float a = s * sqrt_mufu(r2.x);
     float e = ex2(fmaf(a, -kLog2eDt, off));
     v.x = fmaf(a, e, e);
-    a = s * (r2.y * rsqrtf(fmaxf(r2.y, 1e-30f)));
+    a = s * sqrt_mufu(r2.y);
     e = ex2(fmaf(a, -kLog2eDt, off));
     v.y = fmaf(a, e, e);
     return v;
