@@ -95,6 +95,11 @@ struct Ctx {
   // caller's stream by ev_in / ev_out
   cudaStream_t work = nullptr;
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
+  // a second stream inside one product, forked from and joined to the
+  // product's own stream by ev_fork / ev_join (null: no fork).  Sub-contexts
+  // and point sets use their handle's: calls on a handle do not overlap on the host.
+  cudaStream_t aux = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   // concurrent branches of a batched solve each get a sub-context with its
   // own workspace and error word (sub-contexts own no streams or events)
   std::vector<Ctx*> subs;

@@ -122,6 +122,9 @@ cudaError_t sub_context(Ctx& c, size_t k, Ctx** out) {
     if (!s) return cudaErrorMemoryAllocation;
     s->device = c.device;
     s->num_sms = c.num_sms;
+    s->aux = c.aux;
+    s->ev_fork = c.ev_fork;
+    s->ev_join = c.ev_join;
     s->h_counts = c.h_counts;  // a preparation waits for its counts, so the words can be shared
     cudaError_t e = cudaMalloc(&s->d_err, sizeof(int));
     if (!e) e = cudaMemset(s->d_err, 0, sizeof(int));
@@ -288,13 +291,17 @@ krr_status krr_create(krr_handle* out) {
   if (!e) e = cudaStreamCreateWithFlags(&c.work, cudaStreamNonBlocking);
   if (!e) e = cudaEventCreateWithFlags(&c.ev_in, cudaEventDisableTiming);
   if (!e) e = cudaEventCreateWithFlags(&c.ev_out, cudaEventDisableTiming);
+  if (!e) e = cudaStreamCreateWithFlags(&c.aux, cudaStreamNonBlocking);
+  if (!e) e = cudaEventCreateWithFlags(&c.ev_fork, cudaEventDisableTiming);
+  if (!e) e = cudaEventCreateWithFlags(&c.ev_join, cudaEventDisableTiming);
   if (e) {
     cudaGetLastError();
     if (c.d_err) cudaFree(c.d_err);
     if (c.h_status) cudaFreeHost(c.h_status);
-    for (cudaEvent_t ev : {c.ev0, c.ev1, c.ev_in, c.ev_out})
+    for (cudaEvent_t ev : {c.ev0, c.ev1, c.ev_in, c.ev_out, c.ev_fork, c.ev_join})
       if (ev) cudaEventDestroy(ev);
-    if (c.work) cudaStreamDestroy(c.work);
+    for (cudaStream_t s : {c.work, c.aux})
+      if (s) cudaStreamDestroy(s);
     cudaGetLastError();
     delete h;
     return e == cudaErrorMemoryAllocation ? KRR_ERR_OOM : KRR_ERR_CUDA;
@@ -315,8 +322,11 @@ krr_status krr_destroy(krr_handle h) {
   cudaEventDestroy(c.ev1);
   cudaEventDestroy(c.ev_in);
   cudaEventDestroy(c.ev_out);
+  cudaEventDestroy(c.ev_fork);
+  cudaEventDestroy(c.ev_join);
   for (auto ev : c.prof_ev) cudaEventDestroy(ev);
   cudaStreamDestroy(c.work);
+  cudaStreamDestroy(c.aux);
   delete h;
   return KRR_OK;
 }
@@ -546,6 +556,9 @@ krr_status krr_points_create(krr_handle h, const float* X, int64_t N, int d, flo
   Ctx& pc = pts->ctx;
   pc.device = c.device;
   pc.num_sms = c.num_sms;
+  pc.aux = c.aux;
+  pc.ev_fork = c.ev_fork;
+  pc.ev_join = c.ev_join;
   copy_product_options(pc, c);
   cudaError_t e = cudaMalloc(&pc.d_err, sizeof(int));
   if (!e) e = cudaMemsetAsync(pc.d_err, 0, sizeof(int), st);

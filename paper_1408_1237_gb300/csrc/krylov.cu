@@ -328,9 +328,9 @@ __global__ void __launch_bounds__(STEP_T)
 #pragma unroll
   for (int k = 0; k < R; ++k) {
     // the finalize kernel's roundings
-    const double y = fma((double)f.shift, (double)pv[k], __dmul_rn((double)fc[k], sum[k]));
+    const double y = fma((double)f.shift, f2d(pv[k]), __dmul_rn(f2d(fc[k]), sum[k]));
     mp[k] = (float)y;
-    acc += y * (double)pv[k];
+    acc += y * f2d(pv[k]);
   }
   const double inv_rho = t == 0 && rho > 0.0 ? 1.0 / rho : 0.0;
   const double pAp = cluster_sum<true>(acc, buf, slot[0], rank);
@@ -347,7 +347,8 @@ __global__ void __launch_bounds__(STEP_T)
   for (int k = 0; k < R; ++k) {
     zv[k] = fmaf(a, pv[k], zv[k]);
     rv[k] = fmaf(-a, mp[k], rv[k]);
-    acc += (double)rv[k] * (double)rv[k];
+    const double rk = f2d(rv[k]);
+    acc += rk * rk;
   }
   const double rr = cluster_sum<false>(acc, buf, slot[1], rank);
   const bool brk = brk0 || !good;

@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) mvp_dirtc_kernel(const DtParams
       const int c = rt * 8 + 2 * t + (e & 1);
       const int64_t i = row0 + g + 8 * (e >> 1);
       if (c < p.m && i < p.Nt_pad)
-        p.part[((int64_t)blockIdx.y * p.m + c) * p.Nt_pad + i] = (double)S[rt][e] - (double)C[rt][e];
+        p.part[((int64_t)blockIdx.y * p.m + c) * p.Nt_pad + i] = f2d(S[rt][e]) - f2d(C[rt][e]);
     }
 }
 

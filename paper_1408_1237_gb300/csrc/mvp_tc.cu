@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
           if (c >= p.m) continue;
           const int e = 2 * half + cc;
           p.part[((int64_t)blockIdx.y * p.m + c) * p.Nt_pad + i] =
-              (double)S[mt][rt][e] - (double)C[mt][rt][e];
+              f2d(S[mt][rt][e]) - f2d(C[mt][rt][e]);
         }
     }
 }
@@ -669,7 +669,7 @@ __global__ void __launch_bounds__(32 * (SB / (16 * MT))) mvp_tcx_kernel(const Tc
   for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      double v = (double)S[mt][h] - (double)C[mt][h];
+      double v = f2d(S[mt][h]) - f2d(C[mt][h]);
       v += __shfl_xor_sync(0xffffffffu, v, 1);
       v += __shfl_xor_sync(0xffffffffu, v, 2);
       const int64_t i = row0 + mt * 16 + g + 8 * h;
@@ -915,7 +915,7 @@ __global__ void __launch_bounds__(32 * HighD<D>::WARPS) mvp_tch_kernel(const TcP
   for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      double v = (double)S[mt][h] - (double)C[mt][h];
+      double v = f2d(S[mt][h]) - f2d(C[mt][h]);
       v += __shfl_xor_sync(0xffffffffu, v, 1);
       v += __shfl_xor_sync(0xffffffffu, v, 2);
       const int64_t i = row0 + (warp * MT + mt) * 16 + g + 8 * h;
@@ -1366,7 +1366,7 @@ __global__ void __launch_bounds__(umma::THREADS + 32) mvp_umma_kernel(const TcPa
 #pragma unroll
       for (int c = 0; c < YW; ++c) {
         const int col = YW * grp + c;
-        if (col < p.m) p.part[((int64_t)blockIdx.y * p.m + col) * p.Nt_pad + i] = (double)Ssum[c] - (double)Scomp[c];
+        if (col < p.m) p.part[((int64_t)blockIdx.y * p.m + col) * p.Nt_pad + i] = f2d(Ssum[c]) - f2d(Scomp[c]);
       }
     }
   }
@@ -1755,7 +1755,7 @@ __global__ void __launch_bounds__(umma::THREADS + 32, 2) mvp_umx_kernel(const Tc
 #pragma unroll
         for (int c = 0; c < YW; ++c) {
           const int col = YW * grp + c;
-          if (col < p.m) p.part[((int64_t)blockIdx.y * p.m + col) * p.Nt_pad + i] = (double)Ssum[c] - (double)Scomp[c];
+          if (col < p.m) p.part[((int64_t)blockIdx.y * p.m + col) * p.Nt_pad + i] = f2d(Ssum[c]) - f2d(Scomp[c]);
         }
       }
     }
@@ -2054,10 +2054,10 @@ __global__ void __launch_bounds__(uhd::WORKERS + 32) mvp_uhd_kernel(const TcPara
     __syncthreads();
   }
   // the two halves of each row
-  if (!mma_warp && half == 1) red[row] = (double)S - (double)C;
+  if (!mma_warp && half == 1) red[row] = f2d(S) - f2d(C);
   __syncthreads();
   if (!abort_flag && !mma_warp && half == 0 && i < p.Nt_pad)
-    p.part[(int64_t)blockIdx.y * p.Nt_pad + i] = ((double)S - (double)C) + red[row];
+    p.part[(int64_t)blockIdx.y * p.Nt_pad + i] = (f2d(S) - f2d(C)) + red[row];
   umma::fence_before();
   __syncthreads();
   umma::fence_after();
