@@ -77,6 +77,11 @@ struct PointsDev {
 // Targets per super-block.
 constexpr int SB = 256;
 
+// Source tiles (of SB points) that hold points.  The prepared arrays are padded
+// to PAD = 8 tiles; the tiles behind the last point have zero weights and are
+// left out of every product (4,097 points: 17 tiles of 24).
+inline int source_tiles(const PointsDev& S) { return (int)((S.N + SB - 1) / SB); }
+
 // Targets per thread the product kernels use for N targets in d dimensions.
 int mvp_targets_per_thread(int d, int64_t N);
 // Squared radius (scaled units) up to which a warp block uses the expanded form.

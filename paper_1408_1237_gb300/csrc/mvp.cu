@@ -610,8 +610,18 @@ struct Plan {
 };
 
 // scale: the autotuner's factor on the modelled split count (1: the model);
-// setup: a CTA's fixed cost in source tiles.
-Plan make_plan(int64_t nblk, int ntiles, int num_sms, int plan_slots, double scale, double setup = 0.0) {
+// setup: a CTA's fixed cost (launch, target loads, epilogue) in source tiles.
+// Without it the model prefers many splits of a tile or two to a slightly
+// longer last wave: 64 direct-form blocks and 65 tiles got 33 splits of 2
+// (16,385 points, d = 8, f16, 16 columns: 354 us, and 301 with 7 splits of 10).
+// Where a tile is long it hardly counts, and finer splits balance better
+// (Matern, 8 targets per thread, 100,003 points: 3.62 ms with 49 splits of 8
+// tiles, 3.84 with 6 of 66).
+constexpr double SETUP_F32 = 0.3;    // mvp_f32_kernel, per 1 / T (T targets per thread)
+constexpr double SETUP_TCX = 0.1;    // mvp_tcx_kernel
+constexpr double SETUP_MULTI = 0.3;  // mvp_tc_kernel, mvp_umx_kernel
+constexpr double SETUP_DIRTC = 0.5;  // mvp_dirtc_kernel (512 threads, one CTA per SM)
+Plan make_plan(int64_t nblk, int ntiles, int num_sms, int plan_slots, double scale, double setup) {
   const int slots = plan_slots > 0 ? plan_slots : num_sms * 2;
   const int64_t ctas = (nblk + NW - 1) / NW;
   Plan pl;
@@ -725,6 +735,10 @@ cudaError_t dirm_dispatch(const MvpParams& p, int d, int kf, const float* Q, int
   return dirm_dispatch_k<0>(p, d, Q, q_stride, m, T, slot0, pl, st, launch);
 }
 
+Plan f32_plan(const Ctx& c, const PointsDev& Tp, const PointsDev& Sp) {
+  return make_plan(Tp.nblk, source_tiles(Sp), c.num_sms, c.plan_slots, c.split_scale, SETUP_F32 / Tp.T);
+}
+
 // Source splits of the multi-column kernels (one CTA per super-block): the
 // tensor-core kernel over the expanded-form super-blocks, the CUDA-core
 // kernel over the direct-form ones, each planned for its own grid.
@@ -732,8 +746,8 @@ Plan multi_plan_tc(const Ctx& c, const PointsDev& Tp, const PointsDev& Sp, krr_p
   // two CTAs (of 128 targets) per super-block, at most two per SM (tensor memory)
   // one CTA per super-block (mma.sync kernel), or two of 128 targets with at
   // most two per SM (tcgen05 kernel: tensor memory)
-  return make_plan((tc5_on(c, prec, m, Tp) ? 2 : 1) * Tp.h_sb_nexp * NW, (int)(Sp.Npad / TS), c.num_sms,
-                   c.plan_slots, c.split_scale);
+  return make_plan((tc5_on(c, prec, m, Tp) ? 2 : 1) * Tp.h_sb_nexp * NW, source_tiles(Sp), c.num_sms,
+                   c.plan_slots, c.split_scale, SETUP_MULTI);
 }
 // Multi-column products keep the tensor cores to d <= 8 (Gaussian); elsewhere
 // every super-block takes the direct form, whatever its compactness flag.
@@ -749,10 +763,10 @@ bool use_dirtc(const Ctx& c, const PointsDev& Tp) {
 }
 Plan multi_plan_dir(const Ctx& c, const PointsDev& Tp, const PointsDev& Sp) {
   if (use_dirtc(c, Tp))
-    return make_plan((Tp.nsb - multi_nexp(Tp)) * NW, (int)(Sp.Npad / TS), c.num_sms,
-                     c.plan_slots > 0 ? c.plan_slots : c.num_sms, c.split_scale);
-  return make_plan((Tp.nsb - multi_nexp(Tp)) * NW, (int)(Sp.Npad / TS), c.num_sms, c.plan_slots,
-                   c.split_scale);
+    return make_plan((Tp.nsb - multi_nexp(Tp)) * NW, source_tiles(Sp), c.num_sms,
+                     c.plan_slots > 0 ? c.plan_slots : c.num_sms, c.split_scale, SETUP_DIRTC);
+  return make_plan((Tp.nsb - multi_nexp(Tp)) * NW, source_tiles(Sp), c.num_sms, c.plan_slots,
+                   c.split_scale, SETUP_F32);
 }
 
 // The single-column float32 product takes the tensor-core exponent path when
@@ -772,10 +786,10 @@ bool use_tcx(const Ctx& c, const PointsDev& Tp) {
 bool tcx_dir_f32(const PointsDev& Tp) { return Tp.T * 32 == SB; }
 Plan tcx_dir_plan(const Ctx& c, const PointsDev& Tp, const PointsDev& Sp) {
   if (tcx_dir_f32(Tp))
-    return make_plan(Tp.nsb - Tp.h_sb_nexp, (int)(Sp.Npad / TS), c.num_sms, c.plan_slots,
-                     c.split_scale);
-  return make_plan((Tp.nsb - Tp.h_sb_nexp) * NW, (int)(Sp.Npad / TS), c.num_sms, c.plan_slots,
-                   c.split_scale);
+    return make_plan(Tp.nsb - Tp.h_sb_nexp, source_tiles(Sp), c.num_sms, c.plan_slots,
+                     c.split_scale, SETUP_F32 / Tp.T);
+  return make_plan((Tp.nsb - Tp.h_sb_nexp) * NW, source_tiles(Sp), c.num_sms, c.plan_slots,
+                   c.split_scale, SETUP_F32);
 }
 
 Plan tcx_plan(const Ctx& c, const PointsDev& Tp, const PointsDev& Sp) {
@@ -785,17 +799,17 @@ Plan tcx_plan(const Ctx& c, const PointsDev& Tp, const PointsDev& Sp) {
       // resident per SM (two at d = 16: shared and tensor memory); a CTA
       // first builds its 128 target K-vectors (about half a source tile)
       const int occ = Tp.d <= 16 ? 2 : 1;
-      return make_plan(2 * Tp.h_sb_nexp * NW, (int)(Sp.Npad / TS), c.num_sms,
+      return make_plan(2 * Tp.h_sb_nexp * NW, source_tiles(Sp), c.num_sms,
                        c.plan_slots > 0 ? c.plan_slots : occ * c.num_sms, c.split_scale, 0.5);
     }
     // high-dimensional kernel: one CTA per SM (two at d = 16), and a CTA
     // first builds its 256 target K-vectors (about one source tile of work)
     const int occ = Tp.d <= 16 ? 2 : 1;
-    return make_plan(Tp.h_sb_nexp * NW, (int)(Sp.Npad / TS), c.num_sms,
+    return make_plan(Tp.h_sb_nexp * NW, source_tiles(Sp), c.num_sms,
                      c.plan_slots > 0 ? c.plan_slots : occ * c.num_sms, c.split_scale, 1.0);
   }
-  return make_plan(Tp.h_sb_nexp * NW, (int)(Sp.Npad / TS), c.num_sms,
-                   c.plan_slots > 0 ? c.plan_slots : 4 * c.num_sms, c.split_scale);
+  return make_plan(Tp.h_sb_nexp * NW, source_tiles(Sp), c.num_sms,
+                   c.plan_slots > 0 ? c.plan_slots : 4 * c.num_sms, c.split_scale, SETUP_TCX);
 }
 
 // Buffers every product path uses: the factored scale and the dot scratch.
@@ -821,7 +835,7 @@ cudaError_t common_reserve(Ctx& c, const PointsDev& Tp, cudaStream_t st) {
 int route_splits(const Ctx& c, const PointsDev& Tp, const PointsDev& Sp, int m, krr_precision prec) {
   if (m == 1 && prec == KRR_FP32) {
     if (use_tcx(c, Tp)) return std::max(tcx_plan(c, Tp, Sp).splits, tcx_dir_plan(c, Tp, Sp).splits);
-    if (Tp.d <= 8) return make_plan(Tp.nblk, (int)(Sp.Npad / TS), c.num_sms, c.plan_slots, c.split_scale).splits;
+    if (Tp.d <= 8) return f32_plan(c, Tp, Sp).splits;
   }
   int s = multi_plan_dir(c, Tp, Sp).splits;
   if (!multi_direct_only(Tp)) s = std::max(s, multi_plan_tc(c, Tp, Sp, prec, m).splits);
@@ -990,7 +1004,7 @@ cudaError_t mvp_reserve(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, cudaSt
     return dirm_dispatch(p, Tp.d, Tp.kfam, nullptr, 0, 1, SB / 32, Tp.h_sb_nexp, pd, st, false);
   }
   if (Tp.d < 1) return cudaErrorNotSupported;
-  const Plan pl = make_plan(Tp.nblk, (int)(Sp.Npad / TS), c.num_sms, c.plan_slots, c.split_scale);
+  const Plan pl = f32_plan(c, Tp, Sp);
   void* v;
   cudaError_t e;
   const unsigned fin_blocks = (unsigned)((Tp.Npad + 255) / 256);
@@ -1067,7 +1081,7 @@ cudaError_t tcx_path(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, const flo
     p.nblk = Tp.nsb;
     p.xs = Sp.xs;
     p.q = q;
-    p.ntiles = (int)(Sp.Npad / TS);
+    p.ntiles = source_tiles(Sp);
     p.err = c.d_err;
   p.row_lo = c.row_lo;
   p.row_hi = c.row_hi;
@@ -1144,7 +1158,7 @@ cudaError_t mvp_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, const f
   p.nblk = Tp.nblk;
   p.xs = Sp.xs;
   p.q = q;
-  p.ntiles = (int)(Sp.Npad / TS);
+  p.ntiles = source_tiles(Sp);
   p.s = Sp.scale;
   p.active = o.active;
   p.part_stride = Tp.Npad;
@@ -1152,7 +1166,7 @@ cudaError_t mvp_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, const f
   p.row_lo = c.row_lo;
   p.row_hi = c.row_hi;
   if (Tp.d < 1 || Tp.d > 8) return cudaErrorNotSupported;
-  const Plan pl = make_plan(Tp.nblk, p.ntiles, c.num_sms, c.plan_slots, c.split_scale);
+  const Plan pl = f32_plan(c, Tp, Sp);
   cudaError_t e = mvp_reserve(c, Tp, Sp, st);
   if (e) return e;
   void *part, *fac, *dpart, *dcnt;
@@ -1281,7 +1295,7 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, c
   p.tn_exp = Tp.sb_nexp;
   p.nblk = Tp.nsb;
   p.xs = Sp.xs;
-  p.ntiles = (int)(Sp.Npad / TS);
+  p.ntiles = source_tiles(Sp);
   p.err = c.d_err;
   p.row_lo = c.row_lo;
   p.row_hi = c.row_hi;

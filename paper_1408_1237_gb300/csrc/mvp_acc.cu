@@ -645,7 +645,7 @@ struct AccPlan {
 
 // scale: the autotuner's factor on the modelled split count (1: the model).
 AccPlan acc_plan(const PointsDev& P, int num_sms, int plan_slots, int ncols, double scale) {
-  const int ntiles = (int)(P.Npad / TS);
+  const int ntiles = source_tiles(P);
   // one target per thread in the multi-column kernel, ACC_TA otherwise
   const int ta = (ncols > 1 || P.d > 8) ? 1 : ACC_TA;
   const int64_t ctas = (P.N + NT * ta - 1) / (NT * ta);
@@ -758,7 +758,7 @@ cudaError_t mvp_acc_launch(Ctx& c, const PointsDev& P, const float* qh, const fl
   p.qh = qh;
   p.ql = ql;
   p.tbox = P.tbox;
-  p.ntiles = (int)(P.Npad / TS);
+  p.ntiles = source_tiles(P);
   p.err = c.d_err;
   p.k = make_consts();
   // s^2 (Gaussian: log2(e) / (2 sigma^2); Matern: 3 / h^2) and s in

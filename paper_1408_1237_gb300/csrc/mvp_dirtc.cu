@@ -481,7 +481,7 @@ cudaError_t mvp_dirtc_partials(Ctx& c, const PointsDev& T, const PointsDev& S, c
   p.Q = Q;
   p.q_stride = S.Npad;
   p.m = m;
-  p.ntiles = (int)(S.Npad / TS);
+  p.ntiles = source_tiles(S);
   p.tiles_per_split = tiles_per_split;
   p.part = part;
   p.fac = fac;

@@ -2268,7 +2268,7 @@ cudaError_t mvp_tc_partials(Ctx& c, const PointsDev& T, const PointsDev& S, cons
   p.Q = Q;
   p.Ns_pad = S.Npad;
   p.m = m;
-  p.ntiles = (int)(S.Npad / TS);
+  p.ntiles = source_tiles(S);
   p.tiles_per_split = tiles_per_split;
   p.part = part;
   p.fac = fac;
@@ -2306,7 +2306,7 @@ cudaError_t mvp_tcx_partials(Ctx& c, const PointsDev& T, const PointsDev& S, con
   p.Q = q;
   p.Ns_pad = S.Npad;
   p.m = 1;
-  p.ntiles = (int)(S.Npad / TS);
+  p.ntiles = source_tiles(S);
   p.tiles_per_split = tiles_per_split;
   p.part = part;
   p.fac = fac;
@@ -2344,9 +2344,10 @@ cudaError_t mvp_umma_partials(Ctx& c, const PointsDev& T, const PointsDev& S, co
   if (!e && split) e = c.ws.get("umma.ql", sizeof(uint16_t) * umma::YN * TS * (size_t)ntiles, &ql);
   if (e) return e;
   if (!dry) {
-    const unsigned blocks = (unsigned)((ntiles * 512 + 255) / 256);
-    if (bf) q_split_kernel<true><<<blocks, 256, 0, st>>>(Q, m, S.Npad, ntiles, (uint16_t*)qh, nullptr, active);
-    else q_split_kernel<false><<<blocks, 256, 0, st>>>(Q, m, S.Npad, ntiles, (uint16_t*)qh,
+    const int64_t nt = source_tiles(S);
+    const unsigned blocks = (unsigned)((nt * 512 + 255) / 256);
+    if (bf) q_split_kernel<true><<<blocks, 256, 0, st>>>(Q, m, S.Npad, nt, (uint16_t*)qh, nullptr, active);
+    else q_split_kernel<false><<<blocks, 256, 0, st>>>(Q, m, S.Npad, nt, (uint16_t*)qh,
                                                        split ? (uint16_t*)ql : nullptr, active);
     count_launch();
     if ((e = cudaGetLastError())) return e;
@@ -2366,7 +2367,7 @@ cudaError_t mvp_umma_partials(Ctx& c, const PointsDev& T, const PointsDev& S, co
   p.Q = Q;
   p.Ns_pad = S.Npad;
   p.m = m;
-  p.ntiles = (int)(S.Npad / TS);
+  p.ntiles = source_tiles(S);
   p.tiles_per_split = tiles_per_split;
   p.part = part;
   p.fac = fac;
