@@ -222,7 +222,10 @@ krr_status krr_set_option(krr_handle h, int option, int value);
 /* ----------------------------------------------------------- kernel MVP
  * Y = (K_hat + gamma I) Q  (Eqs. 1-3; the weighted kernel sum of Sec. 3.1):
  *     Y[i,c] = sum_j exp(-|x_i - x_j|^2 / (2 sigma^2)) Q[j,c] + gamma Q[i,c]
- * over all N^2 pairs (no cut-off), summed on the fly in O(N) memory.
+ * over all N^2 pairs (no cut-off), summed on the fly in O(N) memory.  (Whole
+ * tiles of pairs whose kernel values come out as exact zeros, below 2^-126 or
+ * below f16's range where the kernel stores them in f16, are not visited: the
+ * sums are those of visiting them, bit for bit.)
  * X: N x d; Q, Y: N x m column-major, 1 <= m <= 64.  Y must not alias X or Q.
  * m = 1 takes one exponential per pair, with the exponent contraction on the
  * tensor cores for compact target blocks and the CUDA-core kernel for the
@@ -417,7 +420,8 @@ typedef struct {
                                accurate product) timed since the last read      */
     double product_ms;      /* their summed device time (CUDA events recorded
                                on the stream each launch ran on)                */
-    double product_pairs;   /* target x source pairs they evaluated, per column */
+    double product_pairs;   /* target x source pairs they covered, per column
+                               (tiles of exact zeros among them)               */
     int tensor_exponent_launches; /* of the timed launches, those that took the
                                tensor-core exponent path (the exponent
                                contraction on the tensor cores, one MUFU.EX2

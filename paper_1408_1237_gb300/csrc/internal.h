@@ -264,9 +264,11 @@ void release_context(Ctx& c);
 cudaError_t prepare_points(Ctx& c, const float* X, int64_t N, int d, float sigma,
                            const char* tag, PointsDev& P, cudaStream_t st);
 // out[i] = in[perm[i]] (float columns, m of them, column stride N / Npad);
-// padded tail of each column set to zero.
+// padded tail of each column set to zero.  qbad (may be null): per tile of SB
+// rows, 1 when a value is not below f16's largest in size (infinities and
+// NaNs among them), else 0.
 cudaError_t gather_sorted(const float* in, int64_t N, int m, const int* perm, int64_t Npad,
-                          float* out, cudaStream_t st);
+                          float* out, cudaStream_t st, int* qbad = nullptr);
 // out[perm[i]] = in[i]
 cudaError_t scatter_orig(const float* in, int64_t Npad, int64_t N, int m, const int* perm,
                          float* out, cudaStream_t st);
@@ -314,6 +316,10 @@ struct MvpOut {
   // but `active` are then ignored): a solver's own kernel consumes the sums
   cudaError_t (*finish)(void* arg, const ProdSums& sums, cudaStream_t st) = nullptr;
   void* finish_arg = nullptr;
+  // per source tile, whether it holds a weight that a zero kernel value does
+  // not cancel (gather_sorted; null: none does, as in the solvers, whose
+  // iteration stops on a product that is not finite wherever it appears)
+  const int* qbad = nullptr;
   // an inner product of a solver's preconditioner, which tolerates rounding:
   // several columns take the tensor-core kernels' less exact form
   bool inner = false;
@@ -365,18 +371,18 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& T, const PointsDev& S, con
 // dry = true only sets the kernel attributes (before any graph capture).
 cudaError_t mvp_tc_partials(Ctx& c, const PointsDev& T, const PointsDev& S, const float* Q, int m,
                             krr_precision prec, bool fine, int splits, int tiles_per_split, double* part,
-                            float* fac, const int* active, cudaStream_t st, bool dry = false);
+                            float* fac, const int* active, const int* qbad, cudaStream_t st, bool dry = false);
 // ---- mvp_tc.cu: single-column float32-grade partial sums of the
 // expanded-form super-blocks (exponent on the tensor cores, EX2 + FMA per
 // pair on the CUDA cores); part: [splits][T.Npad].
 cudaError_t mvp_tcx_partials(Ctx& c, const PointsDev& T, const PointsDev& S, const float* q,
                              int splits, int tiles_per_split, double* part, float* fac,
-                             const int* active, cudaStream_t st, bool dry = false);
+                             const int* active, const int* qbad, cudaStream_t st, bool dry = false);
 // ---- mvp_tc.cu: the same partial sums on the 5th-generation tensor cores
 // (tcgen05.mma, accumulators in tensor memory), two CTAs per super-block.
 cudaError_t mvp_umma_partials(Ctx& c, const PointsDev& T, const PointsDev& S, const float* Q, int m,
                               bool split, bool bf, int splits, int tiles_per_split, double* part,
-                              float* fac, const int* active, cudaStream_t st, bool dry = false);
+                              float* fac, const int* active, const int* qbad, cudaStream_t st, bool dry = false);
 // ---- mvp_dirtc.cu: partial sums of the direct-form super-blocks (slots
 // [slot0, nsb) of T.sb_order, checked against the device count tn_exp) of a
 // multi-column product, d <= 8: kernel values on the CUDA cores, the weighted

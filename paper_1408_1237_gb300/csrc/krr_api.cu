@@ -87,9 +87,12 @@ cudaError_t product_prepared(Ctx& c, const PointsDev& P, const float* dQ, int m,
   void* qs;
   cudaError_t e;
   if ((e = c.ws.get("mvp.qs", sizeof(float) * P.Npad * m, &qs))) return e;
-  if ((e = gather_sorted(dQ, N, m, P.perm, P.Npad, (float*)qs, st))) return e;
+  void* qbad;
+  if ((e = c.ws.get("mvp.qbad", sizeof(int) * (P.Npad / SB), &qbad))) return e;
+  if ((e = gather_sorted(dQ, N, m, P.perm, P.Npad, (float*)qs, st, (int*)qbad))) return e;
   if (m == 1) {
     MvpOut o;
+    o.qbad = (const int*)qbad;
     o.perm = P.perm;
     o.out_orig = dY;
     return mvp_launch(c, P, P, (const float*)qs, (const float*)qs, gamma, prec, o, st);
@@ -102,6 +105,7 @@ cudaError_t product_prepared(Ctx& c, const PointsDev& P, const float* dQ, int m,
     const int mc = std::min(width, m - col0);
     const float* qc = (const float*)qs + (size_t)col0 * P.Npad;
     MvpOut o;
+    o.qbad = (const int*)qbad;
     o.perm = P.perm;
     o.out_orig = dY + (size_t)col0 * N;
     if ((e = mvp_multi_launch(c, P, P, qc, mc, qc, gamma, prec, o, st))) return e;
@@ -652,7 +656,9 @@ krr_status krr_kernel_mvp_rect(krr_handle h, const float* Xt, int64_t Nt, const 
     if ((e = prepare_points(c, dXs, Ns, d, sigma, "pts_s", S, st))) return cuda_error(c, e, fn);
     void* qs;
     if ((e = c.ws.get("mvp.qs", sizeof(float) * S.Npad * m, &qs))) return cuda_error(c, e, fn);
-    if ((e = gather_sorted(dQ, Ns, m, S.perm, S.Npad, (float*)qs, st))) return cuda_error(c, e, fn);
+    void* qbad;
+    if ((e = c.ws.get("mvp.qbad", sizeof(int) * (S.Npad / SB), &qbad))) return cuda_error(c, e, fn);
+    if ((e = gather_sorted(dQ, Ns, m, S.perm, S.Npad, (float*)qs, st, (int*)qbad))) return cuda_error(c, e, fn);
     // columns in as few passes as possible where one pass evaluates each
     // kernel value for all of its columns at less than their single cost
     const bool shared = multi_pays(c, T, m, prec);
@@ -662,6 +668,7 @@ krr_status krr_kernel_mvp_rect(krr_handle h, const float* Xt, int64_t Nt, const 
       const int mc = std::min(width, m - col);
       const float* qc = (const float*)qs + (size_t)col * S.Npad;
       MvpOut o;
+      o.qbad = (const int*)qbad;
       o.perm = T.perm;
       o.out_orig = dY + (size_t)col * Nt;
       e = mc == 1 ? mvp_launch(c, T, S, qc, nullptr, 0.f, prec, o, st)

@@ -997,7 +997,7 @@ cudaError_t mvp_reserve(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, cudaSt
     if ((e = c.ws.get("mvp.partt", sizeof(double) * pt.splits * (size_t)Tp.Npad, &v))) return e;
     if ((e = c.ws.get("mvp.partd", sizeof(double) * pd.splits * (size_t)Tp.Npad, &v))) return e;
     if ((e = mvp_tcx_partials(c, Tp, Sp, nullptr, pt.splits, pt.tiles_per_split, nullptr, nullptr,
-                              nullptr, st, true)))
+                              nullptr, nullptr, st, true)))
       return e;
     MvpParams p{};
     p.nblk = Tp.nsb;
@@ -1019,7 +1019,7 @@ cudaError_t mvp_reserve(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, cudaSt
     if ((e = c.ws.get("mvp.partt", sizeof(double) * pt.splits * (size_t)Tp.Npad, &v))) return e;
     if ((e = c.ws.get("mvp.partd", sizeof(double) * pd.splits * (size_t)Tp.Npad, &v))) return e;
     if ((e = mvp_tcx_partials(c, Tp, Sp, nullptr, pt.splits, pt.tiles_per_split, nullptr, nullptr,
-                              nullptr, st, true)))
+                              nullptr, nullptr, st, true)))
       return e;
     MvpParams p{};
     p.nblk = Tp.nsb;
@@ -1068,7 +1068,7 @@ cudaError_t tcx_path(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, const flo
   cudaEvent_t pev1 = prof_begin(c, Tp, Sp, st);
   if (pev1) c.prof_tensor_exp += 1;
   if ((e = mvp_tcx_partials(c, Tp, Sp, q, pt.splits, pt.tiles_per_split, (double*)partt, (float*)fac,
-                            o.active, st)))
+                            o.active, o.qbad, st)))
     return e;
   if (Tp.nsb > Tp.h_sb_nexp) {
     MvpParams p{};
@@ -1252,10 +1252,10 @@ cudaError_t mvp_multi_reserve(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, 
   if (direct_only) return cudaSuccess;  // no expanded-form blocks: no tensor-core kernel
   if (tc5_on(c, prec, m, Tp))
     return mvp_umma_partials(c, Tp, Sp, nullptr, m, prec == KRR_FP32, prec == KRR_BF16, pt.splits,
-                             pt.tiles_per_split, nullptr, nullptr, nullptr, st, true);
+                             pt.tiles_per_split, nullptr, nullptr, nullptr, nullptr, st, true);
   for (bool fine : {false, true})
     if ((e = mvp_tc_partials(c, Tp, Sp, nullptr, m, prec, fine, pt.splits, pt.tiles_per_split, nullptr, nullptr,
-                             nullptr, st, true)))
+                             nullptr, nullptr, st, true)))
       return e;
   return cudaSuccess;
 }
@@ -1349,9 +1349,9 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, c
   if (nexp > 0) {
     e = tc5_on(c, prec, m, Tp)
             ? mvp_umma_partials(c, Tp, Sp, Q, m, prec == KRR_FP32, prec == KRR_BF16, pt.splits,
-                                pt.tiles_per_split, (double*)part, p.fac, o.active, st)
+                                pt.tiles_per_split, (double*)part, p.fac, o.active, o.qbad, st)
             : mvp_tc_partials(c, Tp, Sp, Q, m, prec, !o.inner, pt.splits, pt.tiles_per_split, (double*)part,
-                              p.fac, o.active, st);
+                              p.fac, o.active, o.qbad, st);
     if (e) return e;
   }
   // direct-form super-blocks: all columns in one launch (the weighted sum

@@ -66,6 +66,86 @@ struct TcParams {
   // sorted target rows computed (shard emulation): whole super-blocks outside
   // [row_lo, row_hi) are skipped
   int64_t row_lo = 0, row_hi = INT64_MAX;
+  // tiles whose kernel values all come out as exact zeros (live_tiles): boxes
+  // of the target super-blocks and of the source tiles, tiles with weights a
+  // zero may not stand for (null: none), and the cut for this kernel's values
+  const float* tbox_t = nullptr;
+  const float* tbox_s = nullptr;
+  const int* qbad = nullptr;
+  float cut = 0.f;
+};
+
+// ---- source tiles that can contribute to a super-block
+// The exponent of a pair is E = |x^_i|^2 - |x^_i - x^_j|^2 with |x^_i|^2 at most
+// the squared half-diagonal R2 of the target box, so the whole tile stays
+// below -cut where the squared distance of the boxes exceeds R2 + cut.  For
+//   cut = 128: 2^E < 2^-126, which ex2.approx.ftz flushes to zero;
+//   cut = 26:  2^E < 2^-25, which rounds to zero in f16, hi and lo
+// (each 1 or 2 beyond the bound, where E's own error is below 0.01).  Such a
+// tile adds exact zeros to sums that a zero leaves as they are, bit for bit,
+// so the CTA neither loads nor evaluates it (2^20 points in the cube, sigma =
+// 0.05: 157 -> 107 ms; 131,072 points x 16 columns 5.9 -> 2.3 ms; 50,021-point
+// mixture 519 -> 357 us; a list that keeps every tile costs 1 to 2 us).  A zero may not stand for the
+// product with an infinite weight (or one that f16 turns into infinity) or
+// for the value of a point that is not finite: such tiles stay (qbad; a box
+// that is not finite compares as near).  The gaps are shortened by a few units
+// in the last place of the coordinates, since the boxes are rounded.
+constexpr float CUT_F32 = 128.f, CUT_F16 = 26.f;
+constexpr int LIVE_WORDS = 256;  // 8192 tiles per CTA; longer ranges keep every tile
+
+// Writes bit r of mask for every live tile t_begin + r, r < nt, and returns
+// their number; blk: the CTA's super-block.  All threads call it.
+template <int D>
+__device__ __forceinline__ int live_tiles(const TcParams& p, int64_t blk, int t_begin, int nt, uint32_t* mask,
+                                          int* count) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if (nt > 32 * LIVE_WORDS) return nt;
+  float c[D], h[D], r2 = 0.f;
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    c[k] = p.tbox_t[blk * 2 * D + k];
+    h[k] = p.tbox_t[blk * 2 * D + D + k];
+    r2 = fmaf(p.s * h[k], p.s * h[k], r2);
+  }
+  if (threadIdx.x == 0) *count = 0;
+  __syncthreads();
+  for (int w = warp; 32 * w < nt; w += nw) {
+    const int r = 32 * w + lane;
+    bool live = false;
+    if (r < nt) {
+      const float* b = p.tbox_s + (int64_t)(t_begin + r) * 2 * D;
+      float d2 = 0.f;
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        const float reach = h[k] + b[D + k];
+        const float gap = fabsf(c[k] - b[k]) - reach - 0x1p-21f * (fabsf(c[k]) + fabsf(b[k]) + reach);
+        const float g = p.s * gap;
+        d2 += gap > 0.f ? g * g : gap - gap;  // 0, or NaN from a box that is not finite
+      }
+      live = !(d2 - r2 > p.cut) || (p.qbad && p.qbad[t_begin + r]);
+    }
+    const uint32_t m = __ballot_sync(0xffffffffu, live);
+    if (lane == 0) {
+      mask[w] = m;
+      atomicAdd(count, __popc(m));
+    }
+  }
+  __syncthreads();
+  return *count;
+}
+
+// The live tiles in order, for the thread that issues the copies.
+struct LiveIter {
+  const uint32_t* mask;  // null: every tile
+  int next = 0;
+  uint32_t bits = 0;
+  __device__ __forceinline__ int pop() {  // the next live r (there is one)
+    if (!mask) return next++;
+    while (!bits) bits = mask[next++];
+    const int b = __ffs(bits) - 1;
+    bits &= bits - 1;
+    return 32 * (next - 1) + b;
+  }
 };
 
 // Terms of the split exponent: 4 (Ah Bh + Ah Bl + Al Bh + Al Bl) when 4(D+1)
@@ -177,6 +257,8 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
   const int g = lane >> 2, t = lane & 3;
   __shared__ __align__(8) uint64_t bars[RS];
   __shared__ volatile int abort_flag;
+  __shared__ uint32_t live[LIVE_WORDS];
+  __shared__ int live_n;
   if (p.active && *p.active == 0) return;
   const int64_t nexp = *p.tn_exp;
   if ((int64_t)blockIdx.x >= nexp) return;  // direct-form blocks: CUDA-core kernel
@@ -226,7 +308,9 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
   }
 
   const int t_begin = blockIdx.y * p.tiles_per_split;
-  const int nt = min(p.ntiles, t_begin + p.tiles_per_split) - t_begin;
+  const int nt_all = min(p.ntiles, t_begin + p.tiles_per_split) - t_begin;
+  const int nt = live_tiles<D>(p, blk, t_begin, nt_all, live, &live_n);  // this CTA's tiles
+  LiveIter tiles{nt_all > 32 * LIVE_WORDS ? nullptr : live};
 
   // acc: P Q of the tile (SPLIT 2: Ph Qh of the current FOLD sources);
   // low: SPLIT 2, Pl Qh + Ph Ql of the tile
@@ -242,7 +326,7 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
 
   auto issue = [&](int r) {
     const int stage = r % RS;
-    const int64_t tile = t_begin + r;
+    const int64_t tile = t_begin + tiles.pop();
     float* dst = raw + stage * raw_floats;
     mbar_arrive_expect_tx(&bars[stage], (uint32_t)raw_floats * 4);
     bulk_g2s(dst, p.xs + tile * (int64_t)D * TS, D * TS * 4, &bars[stage]);
@@ -476,6 +560,8 @@ __global__ void __launch_bounds__(32 * (SB / (16 * MT))) mvp_tcx_kernel(const Tc
   const int g = lane >> 2, t = lane & 3;
   __shared__ __align__(8) uint64_t bars[RS];
   __shared__ volatile int abort_flag;
+  __shared__ uint32_t live[LIVE_WORDS];
+  __shared__ int live_n;
   if (p.active && *p.active == 0) return;
   const int64_t nexp = *p.tn_exp;
   if ((int64_t)blockIdx.x >= nexp) return;
@@ -522,7 +608,9 @@ __global__ void __launch_bounds__(32 * (SB / (16 * MT))) mvp_tcx_kernel(const Tc
   }
 
   const int t_begin = blockIdx.y * p.tiles_per_split;
-  const int nt = min(p.ntiles, t_begin + p.tiles_per_split) - t_begin;
+  const int nt_all = min(p.ntiles, t_begin + p.tiles_per_split) - t_begin;
+  const int nt = live_tiles<D>(p, blk, t_begin, nt_all, live, &live_n);  // this CTA's tiles
+  LiveIter tiles{nt_all > 32 * LIVE_WORDS ? nullptr : live};
   float2 acc[MT][2], acc2[MT][2];
   float S[MT][2], C[MT][2];
 #pragma unroll
@@ -535,7 +623,7 @@ __global__ void __launch_bounds__(32 * (SB / (16 * MT))) mvp_tcx_kernel(const Tc
 
   auto issue = [&](int r) {
     const int stage = r % RS;
-    const int64_t tile = t_begin + r;
+    const int64_t tile = t_begin + tiles.pop();
     float* dst = raw + stage * RAW;
     mbar_arrive_expect_tx(&bars[stage], (uint32_t)RAW * 4);
     bulk_g2s(dst, p.xs + tile * (int64_t)D * TS, D * TS * 4, &bars[stage]);
@@ -1454,6 +1542,8 @@ __global__ void __launch_bounds__(umma::THREADS + 32, 2) mvp_umx_kernel(const Tc
   __shared__ __align__(8) uint64_t dbar;         // after an abort: the MMAs issued are complete
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
+  __shared__ uint32_t live[LIVE_WORDS];
+  __shared__ int live_n;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
   const bool mma_warp = warp == NCW;
@@ -1536,11 +1626,13 @@ __global__ void __launch_bounds__(umma::THREADS + 32, 2) mvp_umx_kernel(const Tc
   static_assert(NBUF * NC + 2 * YW2 <= TMEM_COLS, "tensor-memory columns");
   const uint32_t y_col = NBUF * NC;
   const int t_begin = blockIdx.y * p.tiles_per_split;
-  const int nt = min(p.ntiles, t_begin + p.tiles_per_split) - t_begin;
+  const int nt_all = min(p.ntiles, t_begin + p.tiles_per_split) - t_begin;
+  const int nt = live_tiles<D>(p, blk, t_begin, nt_all, live, &live_n);  // this CTA's tiles
+  LiveIter tiles{nt_all > 32 * LIVE_WORDS ? nullptr : live};
 
   auto issue = [&](int r) {
     const int stage = r % URS;
-    const int64_t tile = t_begin + r;
+    const int64_t tile = t_begin + tiles.pop();
     unsigned char* dst = stages + stage * SBYTES;
     mbar_arrive_expect_tx(&bars[stage], SBYTES);
     bulk_g2s(dst, p.xs + tile * (int64_t)D * TS, D * TS * 4, &bars[stage]);
@@ -2252,7 +2344,7 @@ cudaError_t dispatch_prec(const TcParams& p, int splits, krr_precision prec, boo
 
 cudaError_t mvp_tc_partials(Ctx& c, const PointsDev& T, const PointsDev& S, const float* Q, int m,
                             krr_precision prec, bool fine, int splits, int tiles_per_split, double* part,
-                            float* fac, const int* active, cudaStream_t st, bool dry) {
+                            float* fac, const int* active, const int* qbad, cudaStream_t st, bool dry) {
   if (m < 1 || m > 16) return cudaErrorNotSupported;
   TcParams p{};
   p.xt = T.xs;
@@ -2277,6 +2369,10 @@ cudaError_t mvp_tc_partials(Ctx& c, const PointsDev& T, const PointsDev& S, cons
   p.row_hi = c.row_hi;
   p.s = S.scale;
   p.active = active;
+  p.tbox_t = T.tbox;
+  p.tbox_s = S.tbox;
+  p.qbad = qbad;
+  p.cut = prec == KRR_BF16 ? CUT_F32 : CUT_F16;  // P as f16 (hi + lo)
   switch (T.d) {
     case 1: return dispatch_prec<1>(p, splits, prec, fine, st, dry);
     case 2: return dispatch_prec<2>(p, splits, prec, fine, st, dry);
@@ -2292,7 +2388,7 @@ cudaError_t mvp_tc_partials(Ctx& c, const PointsDev& T, const PointsDev& S, cons
 
 cudaError_t mvp_tcx_partials(Ctx& c, const PointsDev& T, const PointsDev& S, const float* q,
                              int splits, int tiles_per_split, double* part, float* fac,
-                             const int* active, cudaStream_t st, bool dry) {
+                             const int* active, const int* qbad, cudaStream_t st, bool dry) {
   TcParams p{};
   p.xt = T.xs;
   p.Nt = T.N;
@@ -2315,6 +2411,10 @@ cudaError_t mvp_tcx_partials(Ctx& c, const PointsDev& T, const PointsDev& S, con
   p.row_hi = c.row_hi;
   p.s = S.scale;
   p.active = active;
+  p.tbox_t = T.tbox;
+  p.tbox_s = S.tbox;
+  p.qbad = qbad;
+  p.cut = CUT_F32;
   switch (T.d) {
     case 1: return tcx_launch_typed<1>(p, splits, st, dry);
     case 2: return tcx_launch_typed<2>(p, splits, st, dry);
@@ -2334,7 +2434,7 @@ cudaError_t mvp_tcx_partials(Ctx& c, const PointsDev& T, const PointsDev& S, con
 
 cudaError_t mvp_umma_partials(Ctx& c, const PointsDev& T, const PointsDev& S, const float* Q, int m,
                               bool split, bool bf, int splits, int tiles_per_split, double* part,
-                              float* fac, const int* active, cudaStream_t st, bool dry) {
+                              float* fac, const int* active, const int* qbad, cudaStream_t st, bool dry) {
   if (m < 1 || m > umma::YN) return cudaErrorNotSupported;
   // the weights pre-split per source tile (workspace sized here, also in a
   // dry run, so that a captured launch allocates nothing)
@@ -2376,6 +2476,10 @@ cudaError_t mvp_umma_partials(Ctx& c, const PointsDev& T, const PointsDev& S, co
   p.row_hi = c.row_hi;
   p.s = S.scale;
   p.active = active;
+  p.tbox_t = T.tbox;
+  p.tbox_s = S.tbox;
+  p.qbad = qbad;
+  p.cut = bf ? CUT_F32 : CUT_F16;
   switch (T.d) {
     case 1: return umma_dispatch<1>(p, splits, split, bf, c.tcgen05_kind, st, dry);
     case 2: return umma_dispatch<2>(p, splits, split, bf, c.tcgen05_kind, st, dry);

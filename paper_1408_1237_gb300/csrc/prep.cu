@@ -427,16 +427,20 @@ __global__ void __launch_bounds__(TS)
   const int64_t i = tile * TS + tid;
   const float* row = X + (int64_t)perm[i < N ? i : N - 1] * d_in;
   float* dst = o.xs + tile * (int64_t)d * TS + tid;
+  bool finite = true;
   for (int k = 0; k < d; ++k) {
     const float v = k < d_in ? row[k] : 0.f;  // padded coordinates: 0
     dst[(int64_t)k * TS] = v;
+    finite = finite && isfinite(v);
     const float lo = warp_min(v), hi = warp_max(v);
     if (lane == 0) {
       wlo[warp][k] = lo;
       whi[warp][k] = hi;
     }
   }
-  __syncthreads();
+  // min and max pass over NaN: the box of a tile with a coordinate that is not
+  // finite is NaN (near to everything)
+  const bool tile_finite = __syncthreads_and(finite);
   // the tile's box (and super-block centre), then each group of T warps
   for (int k = tid; k < d; k += TS) {
     float lo = wlo[0][k], hi = whi[0][k];
@@ -446,7 +450,7 @@ __global__ void __launch_bounds__(TS)
     }
     const float c = 0.5f * (lo + hi);
     tctr[k] = c;
-    o.tbox[tile * 2 * d + k] = c;
+    o.tbox[tile * 2 * d + k] = tile_finite ? c : NAN;
     o.tbox[tile * 2 * d + d + k] = 0.5f * (hi - lo);
     if (tile < nsb) o.sb_ctr[tile * d + k] = c;
   }
@@ -492,12 +496,22 @@ __global__ void __launch_bounds__(TS)
   }
 }
 
-__global__ void gather_kernel(const float* __restrict__ in, int64_t N, int m,
-                              const int* __restrict__ perm, int64_t Npad, float* __restrict__ out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= Npad) return;
+// (Npad is a multiple of the block: no thread leaves early)
+__global__ void __launch_bounds__(TS)
+    gather_kernel(const float* __restrict__ in, int64_t N, int m, const int* __restrict__ perm, int64_t Npad,
+                  float* __restrict__ out, int* __restrict__ qbad) {
+  const int64_t i = (int64_t)blockIdx.x * TS + threadIdx.x;
   const int64_t p = i < N ? perm[i] : -1;
-  for (int c = 0; c < m; ++c) out[(int64_t)c * Npad + i] = p >= 0 ? in[(int64_t)c * N + p] : 0.f;
+  bool bad = false;
+  for (int c = 0; c < m; ++c) {
+    const float v = p >= 0 ? in[(int64_t)c * N + p] : 0.f;
+    out[(int64_t)c * Npad + i] = v;
+    bad |= !(fabsf(v) < 65504.f);
+  }
+  if (qbad) {
+    const int any = __syncthreads_or(bad);
+    if (threadIdx.x == 0) qbad[blockIdx.x] = any ? 1 : 0;
+  }
 }
 
 __global__ void scatter_kernel(const float* __restrict__ in, int64_t Npad, int64_t N, int m,
@@ -600,9 +614,9 @@ cudaError_t cluster_sort(const uint32_t* keys, int N, int key_bits, int* perm, c
 }  // namespace
 
 cudaError_t gather_sorted(const float* in, int64_t N, int m, const int* perm, int64_t Npad,
-                          float* out, cudaStream_t st) {
+                          float* out, cudaStream_t st, int* qbad) {
   if (Npad == 0) return cudaSuccess;
-  gather_kernel<<<blocks_for(Npad, 256), 256, 0, st>>>(in, N, m, perm, Npad, out); count_launch();
+  gather_kernel<<<blocks_for(Npad, TS), TS, 0, st>>>(in, N, m, perm, Npad, out, qbad); count_launch();
   return cudaGetLastError();
 }
 
