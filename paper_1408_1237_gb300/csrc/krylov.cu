@@ -304,13 +304,19 @@ __global__ void __launch_bounds__(STEP_T)
   double sum[R];
 #pragma unroll
   for (int k = 0; k < R; ++k) {
-    const int64_t i0 = (int64_t)(k * STEP_CL + rank) * STEP_T, i = i0 + t;
+    const int64_t i = (int64_t)(k * STEP_CL + rank) * STEP_T + t;
     pv[k] = rv[k] = zv[k] = mp[k] = fc[k] = 0.f;
     sum[k] = 0.0;
     if (i >= f.Npad) continue;
     pv[k] = p[co + i];
     rv[k] = r[co + i];
     zv[k] = z[co + i];
+  }
+  pdl_wait();  // the product's sums
+  pdl_trigger();
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    const int64_t i0 = (int64_t)(k * STEP_CL + rank) * STEP_T, i = i0 + t;
     if (i >= f.N) continue;
     fc[k] = f.fac[i];
     const bool second = f.sb_flag && f.sb_flag[i0 / SB] == 0;
@@ -980,13 +986,16 @@ struct Solver {
     cfg.gridDim = dim3(STEP_CL, (unsigned)s.mc);
     cfg.blockDim = dim3(STEP_T);
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = STEP_CL;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    // (a product of several columns or in 16 bits may end in a join of streams)
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = s.mc == 1 && s.inner_prec == KRR_FP32 ? 2 : 1;
     const int64_t rows = (s.Np + STEP_CL * STEP_T - 1) / (STEP_CL * STEP_T);  // per thread
     auto* kernel = rows <= 1 ? cg_step_kernel<1> : rows <= 2 ? cg_step_kernel<2>
                    : rows <= 4 ? cg_step_kernel<4> : cg_step_kernel<8>;

@@ -103,13 +103,18 @@ __device__ __forceinline__ void transform_tile(const float* __restrict__ rs, flo
   }
 }
 
+// Sources per unrolled step are 4 times this: with one target per thread the
+// instruction chains of several sources have to fill the pipes.
+template <int T>
+constexpr int f32_unroll() { return T == 1 ? 8 : 2; }
+
 template <int D, int T>
 __device__ __forceinline__ void compute_expanded(const float* __restrict__ cb,
                                                  const float2 (&tx)[T][D], float2 (&acc)[T]) {
   const float* cX = cb;
   const float* cB = cb + D * TS;
   const float* cQ = cb + (D + 1) * TS;
-#pragma unroll 2
+#pragma unroll f32_unroll<T>()
   for (int j = 0; j < TS; j += 4) {
     float4 xk[D];
 #pragma unroll
@@ -152,7 +157,7 @@ __device__ __forceinline__ void compute_direct(const float* __restrict__ cb,
   const float* cQ = cb + (D + 1) * TS;
   const float2 ns2 = make_float2(-s2, -s2);
   const float2 sv = make_float2(s, s), nl2e = make_float2(-kLog2e, -kLog2e);
-#pragma unroll 2
+#pragma unroll f32_unroll<T>()
   for (int j = 0; j < TS; j += 4) {
     float4 xk[D];
 #pragma unroll
@@ -205,7 +210,6 @@ __global__ void __launch_bounds__(NT, 2) mvp_f32_kernel(const MvpParams p) {
   float* wbuf = smem + RS * kRawFloats + warp * kWbFloats;  // this warp's (D+2) * TS
   __shared__ __align__(8) uint64_t bars[RS];
   __shared__ volatile int abort_flag;
-  if (p.active && *p.active == 0) return;
 
   // ---- this warp's target block
   const int64_t slot = p.slot0 + (int64_t)blockIdx.x * NW + warp;
@@ -240,6 +244,11 @@ __global__ void __launch_bounds__(NT, 2) mvp_f32_kernel(const MvpParams p) {
     }
     r2[u] = a;
   }
+  // up to here only prepared points were read: this part overlaps the kernel
+  // before it (which wrote q and the flag, and read the last sums)
+  pdl_wait();
+  if (p.active && *p.active == 0) return;
+  pdl_trigger();
   if (blockIdx.y == 0 && work) {
 #pragma unroll
     for (int u = 0; u < T; ++u) {
@@ -485,6 +494,7 @@ struct FinParams : ProdSums {
 __global__ void __launch_bounds__(256) mvp_finalize_kernel(const FinParams f) {
   __shared__ double red[8];
   __shared__ bool is_last;
+  pdl_wait();
   if (f.o.active && *f.o.active == 0) return;
   // column blockIdx.y: its vectors are Npad (original order: N) apart, its
   // scalars state_stride bytes apart
@@ -541,6 +551,14 @@ __global__ void __launch_bounds__(256) mvp_finalize_kernel(const FinParams f) {
   }
 }
 
+// A row costs one FP64 addition per source split, and an SM adds two per clock:
+// without the dot product's block sums, blocks of 64 rows spread a small
+// product over more SMs.
+cudaError_t launch_finalize(const FinParams& f, int m, cudaStream_t st) {
+  const int threads = f.o.dot ? 256 : 64;
+  return launch_pdl(mvp_finalize_kernel, dim3((unsigned)((f.Npad + threads - 1) / threads), (unsigned)m), threads, 0, st, f);
+}
+
 template <int D>
 constexpr size_t smem_bytes() {
   return sizeof(float) * (raw_stages<D>() * (D + 1) * TS + NW * (D + 2) * TS);
@@ -565,8 +583,7 @@ cudaError_t launch_typed(const MvpParams& p, int splits, cudaStream_t st) {
   cudaError_t e = set_attr<D, T, KF>();
   if (e) return e;
   dim3 grid((unsigned)std::max<int64_t>(1, (p.nblk - p.slot0 + NW - 1) / NW), (unsigned)splits);
-  mvp_f32_kernel<D, T, KF><<<grid, NT, smem_bytes<D>(), st>>>(p); count_launch();
-  return cudaGetLastError();
+  return launch_pdl(mvp_f32_kernel<D, T, KF>, grid, NT, smem_bytes<D>(), st, p);
 }
 
 // Split count minimising the makespan ceil(blocks*S/slots) * (ceil(tiles/S) +
@@ -1128,8 +1145,7 @@ cudaError_t tcx_path(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, const flo
   f.row_lo = c.row_lo;
   f.row_hi = c.row_hi;
   if (o.finish) return o.finish(o.finish_arg, f, st);
-  mvp_finalize_kernel<<<fin_blocks, 256, 0, st>>>(f); count_launch();
-  return cudaGetLastError();
+  return launch_finalize(f, 1, st);
 }
 
 }  // namespace
@@ -1211,8 +1227,7 @@ cudaError_t mvp_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, const f
   f.row_lo = c.row_lo;
   f.row_hi = c.row_hi;
   if (o.finish) return o.finish(o.finish_arg, f, st);
-  mvp_finalize_kernel<<<fin_blocks, 256, 0, st>>>(f); count_launch();
-  return cudaGetLastError();
+  return launch_finalize(f, 1, st);
 }
 
 cudaError_t mvp_multi_reserve(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, int m,
@@ -1392,8 +1407,7 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, c
   f.row_lo = c.row_lo;
   f.row_hi = c.row_hi;
   if (o.finish) return o.finish(o.finish_arg, f, st);
-  mvp_finalize_kernel<<<dim3(fin_blocks, (unsigned)m), 256, 0, st>>>(f); count_launch();
-  return cudaGetLastError();
+  return launch_finalize(f, m, st);
 }
 
 }  // namespace krr

@@ -500,6 +500,7 @@ __global__ void __launch_bounds__(TS)
 __global__ void __launch_bounds__(TS)
     gather_kernel(const float* __restrict__ in, int64_t N, int m, const int* __restrict__ perm, int64_t Npad,
                   float* __restrict__ out, int* __restrict__ qbad) {
+  pdl_trigger();  // a product kernel reads only prepared points before its wait
   const int64_t i = (int64_t)blockIdx.x * TS + threadIdx.x;
   const int64_t p = i < N ? perm[i] : -1;
   bool bad = false;
