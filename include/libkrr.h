@@ -234,9 +234,10 @@ krr_status krr_set_option(krr_handle h, int option, int value);
  * prec: KRR_FP32 (max relative error per element, against the FP64 sum
  * scaled by sum_j |Q_jc| K_hat_ij + gamma |Q_ic|, below 1e-5) or KRR_BF16 /
  * KRR_FP16 (reduced-precision kernel values, float32 accumulation).
- * The call waits briefly for the point preparation (Hilbert sort and block
- * metadata) to read the block counts that size the product grids; the
- * product itself is asynchronous on device arrays. */
+ * The call may wait briefly for the point preparation (Hilbert sort and block
+ * metadata) to read the block counts that size the product grids (single
+ * columns in float32 of up to 16384 points up to 8 dimensions do not need
+ * them); the product itself is asynchronous on device arrays. */
 krr_status krr_kernel_mvp(krr_handle h, const float* X, int64_t N, int d,
                           float sigma, float gamma, const float* Q, int m,
                           float* Y, krr_precision prec, void* stream);

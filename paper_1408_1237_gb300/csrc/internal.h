@@ -70,8 +70,10 @@ struct PointsDev {
   int* sb_order = nullptr;
   int* sb_nexp = nullptr;
   int* sb_flag = nullptr;  // nsb flags: 1 = expanded form
-  // host copies of *n_exp and *sb_nexp (read once by prepare_points)
+  // host copies of *n_exp and *sb_nexp (read once by prepare_points; without
+  // the read, which waits, only mvp_whole_launch may follow)
   int64_t h_nexp = 0, h_sb_nexp = 0;
+  bool counts_read = false;
 };
 
 // Targets per super-block.
@@ -262,7 +264,7 @@ void release_context(Ctx& c);
 // tile-blocked structure-of-arrays copy.  `tag` names the workspace slots.
 // Under c.morton they are sorted in Morton order.
 cudaError_t prepare_points(Ctx& c, const float* X, int64_t N, int d, float sigma,
-                           const char* tag, PointsDev& P, cudaStream_t st);
+                           const char* tag, PointsDev& P, cudaStream_t st, bool read_counts = true);
 // out[i] = in[perm[i]] (float columns, m of them, column stride N / Npad);
 // padded tail of each column set to zero.  qbad (may be null): per tile of SB
 // rows, 1 when a value is not below f16's largest in size (infinities and
@@ -392,6 +394,11 @@ cudaError_t mvp_dirtc_partials(Ctx& c, const PointsDev& T, const PointsDev& S, c
                                krr_precision prec, int splits, int tiles_per_split, int64_t slot0,
                                const int* tn_exp, double* part, float* fac, const int* active,
                                bool fine, cudaStream_t st, bool dry = false);
+// The whole single-column float32 product of a small square point set in one
+// launch, Q and Y in the caller's order: whether it applies, and the launch.
+bool mvp_whole_fits(const Ctx& c, int64_t N, int d, krr_precision prec);
+cudaError_t mvp_whole_launch(Ctx& c, const PointsDev& P, const float* Q, float shift, float* Y, cudaStream_t st);
+
 // Whether m columns of a product over the targets T cost less in one pass
 // (mvp_multi_launch) than as m single-column products.
 bool multi_pays(const Ctx& c, const PointsDev& T, int m, krr_precision prec);

@@ -74,6 +74,15 @@ struct MvpParams {
   int64_t slot0;        // first block slot of the grid (blocks before it are not processed)
   // sorted target rows computed (shard emulation): blocks outside are skipped
   int64_t row_lo = 0, row_hi = INT64_MAX;
+  // whole product in this launch (mvp_f32_kernel): weights and results in the
+  // caller's order through perm, and the last split of a CTA's targets to
+  // arrive (tick[blockIdx.x]) adds the splits: y = K_hat q + shift q
+  const float* q_orig = nullptr;
+  const int* perm = nullptr;
+  unsigned* tick = nullptr;
+  float* y_orig = nullptr;
+  float shift = 0.f;
+  bool pdl = true;  // (host) the points' preparation is complete: launch as a programmatic dependent
 };
 
 // Warp-cooperative transform of one raw source tile for this warp's centre:
@@ -199,7 +208,8 @@ __device__ __forceinline__ void compute_direct(const float* __restrict__ cb,
   }
 }
 
-template <int D, int T, int KF>
+// WHOLE: the whole product of a small point set (MvpParams::q_orig)
+template <int D, int T, int KF, bool WHOLE>
 __global__ void __launch_bounds__(NT, 2) mvp_f32_kernel(const MvpParams p) {
   constexpr int RS = raw_stages<D>();
   constexpr uint32_t kRawFloats = (D + 1) * TS;
@@ -274,10 +284,16 @@ __global__ void __launch_bounds__(NT, 2) mvp_f32_kernel(const MvpParams p) {
     const int stage = r % RS;
     const int64_t tile = t_begin + r;
     float* dst = raw + stage * kRawFloats;
-    mbar_arrive_expect_tx(&bars[stage], kRawFloats * 4);
+    mbar_arrive_expect_tx(&bars[stage], (WHOLE ? D * TS : kRawFloats) * 4);
     bulk_g2s(dst, p.xs + tile * (int64_t)D * TS, D * TS * 4, &bars[stage]);
-    bulk_g2s(dst + D * TS, p.q + tile * (int64_t)TS, TS * 4, &bars[stage]);
+    if (!WHOLE) bulk_g2s(dst + D * TS, p.q + tile * (int64_t)TS, TS * 4, &bars[stage]);
   };
+  // weight of source tid of tile r, in the caller's order (whole product)
+  auto load_q = [&](int r) {
+    const int64_t j = (int64_t)(t_begin + r) * TS + tid;
+    return r < nt && j < p.Nt ? p.q_orig[p.perm[j]] : 0.f;
+  };
+  float qn = WHOLE ? load_q(0) : 0.f;
 
   if (tid == 0) {
     abort_flag = 0;
@@ -298,6 +314,11 @@ __global__ void __launch_bounds__(NT, 2) mvp_f32_kernel(const MvpParams p) {
     }
     // warp-uniform outcome: a lane that gave up takes its whole warp with it
     const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bars[r % RS], (r / RS) & 1));
+    if (WHOLE) {  // this stage's weight row is written by the threads only
+      raw[(r % RS) * kRawFloats + D * TS + tid] = qn;
+      qn = load_q(r + 1);
+      __syncthreads();
+    }
     if (!ok) {
       abort_flag = 1;
       if (lane == 0) atomicExch(p.err, DEV_TIMEOUT);
@@ -322,6 +343,8 @@ __global__ void __launch_bounds__(NT, 2) mvp_f32_kernel(const MvpParams p) {
     if (tid == 0)
       for (int r = 0; r < issued; ++r) mbar_wait_bounded(&bars[r % RS], (r / RS) & 1);
     __syncthreads();
+    // the count of arrivals stays whole (the error word tells of the loss)
+    if (WHOLE && tid == 0 && atomicAdd(&p.tick[blockIdx.x], 1u) == gridDim.y - 1) p.tick[blockIdx.x] = 0u;
     return;
   }
 
@@ -332,6 +355,27 @@ __global__ void __launch_bounds__(NT, 2) mvp_f32_kernel(const MvpParams p) {
       const int64_t i = blk * 32 * T + lane + 32 * u;
       if (i < p.Nt_pad) part[i] = f2d(sum[u]) - f2d(comp[u]);
     }
+  }
+  if (!WHOLE) return;
+  // the last split to arrive reads every split's sums, in order
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) abort_flag = atomicAdd(&p.tick[blockIdx.x], 1u) == gridDim.y - 1;
+  __syncthreads();
+  if (!abort_flag) return;
+  __threadfence();
+  if (tid == 0) p.tick[blockIdx.x] = 0u;
+  if (!work) return;
+#pragma unroll
+  for (int u = 0; u < T; ++u) {
+    const int64_t i = blk * 32 * T + lane + 32 * u;
+    if (i >= p.Nt) continue;
+    double v = 0.0;
+#pragma unroll 8
+    for (int sp = 0; sp < (int)gridDim.y; ++sp) v += __ldcg(p.part + (int64_t)sp * p.part_stride + i);
+    const int64_t o = p.perm[i];
+    const double yi = fma((double)p.shift, f2d(p.q_orig[o]), __dmul_rn(f2d(expanded ? exp2f(-r2[u]) : 1.f), v));
+    p.y_orig[o] = (float)yi;
   }
 }
 
@@ -565,25 +609,27 @@ constexpr size_t smem_bytes() {
 }
 
 // Dynamic shared-memory opt-in, once per kernel instance and device.
-template <int D, int T, int KF>
+template <int D, int T, int KF, bool WHOLE = false>
 cudaError_t set_attr() {
   static bool done[128] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 128 && done[dev]) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(mvp_f32_kernel<D, T, KF>,
+  cudaError_t e = cudaFuncSetAttribute(mvp_f32_kernel<D, T, KF, WHOLE>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem_bytes<D>());
   if (!e && dev < 128) done[dev] = true;
   return e;
 }
 
-template <int D, int T, int KF>
+template <int D, int T, int KF, bool WHOLE = false>
 cudaError_t launch_typed(const MvpParams& p, int splits, cudaStream_t st) {
-  cudaError_t e = set_attr<D, T, KF>();
+  cudaError_t e = set_attr<D, T, KF, WHOLE>();
   if (e) return e;
   dim3 grid((unsigned)std::max<int64_t>(1, (p.nblk - p.slot0 + NW - 1) / NW), (unsigned)splits);
-  return launch_pdl(mvp_f32_kernel<D, T, KF>, grid, NT, smem_bytes<D>(), st, p);
+  if (p.pdl) return launch_pdl(mvp_f32_kernel<D, T, KF, WHOLE>, grid, NT, smem_bytes<D>(), st, p);
+  mvp_f32_kernel<D, T, KF, WHOLE><<<grid, NT, smem_bytes<D>(), st>>>(p); count_launch();
+  return cudaGetLastError();
 }
 
 // Split count minimising the makespan ceil(blocks*S/slots) * (ceil(tiles/S) +
@@ -662,6 +708,7 @@ template <int D, int KF = 0>
 cudaError_t dispatch_T(MvpParams p, int T, const Plan& pl, cudaStream_t st) {
   constexpr int TL = large_T<D>();
   p.tiles_per_split = pl.tiles_per_split;
+  if (p.q_orig) return T == 1 ? launch_typed<D, 1, KF, true>(p, pl.splits, st) : cudaErrorNotSupported;
   if (T == TL) return launch_typed<D, TL, KF>(p, pl.splits, st);
   if (T == 1) return launch_typed<D, 1, KF>(p, pl.splits, st);
   return cudaErrorNotSupported;
@@ -1228,6 +1275,58 @@ cudaError_t mvp_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, const f
   f.row_hi = c.row_hi;
   if (o.finish) return o.finish(o.finish_arg, f, st);
   return launch_finalize(f, 1, st);
+}
+
+// One launch instead of gather, product and finalize.  With few points the
+// three are launch latency and the host's three calls (4,096 prepared points:
+// 27 us a product and 19 with one); each CTA gathers the weights of its
+// tiles itself, which above WHOLE_MAX_N costs more than the gather.
+constexpr int64_t WHOLE_MAX_N = 16384;
+
+bool mvp_whole_fits(const Ctx& c, int64_t N, int d, krr_precision prec) {
+  // (fewer super-blocks than SMs: the tensor-core exponent path is out)
+  return prec == KRR_FP32 && d <= 8 && N <= WHOLE_MAX_N && mvp_targets_per_thread(d, N) == 1 &&
+         (N + SB - 1) / SB < c.num_sms && !c.autotune && !c.profiling && !c.ws.fixed;
+}
+
+cudaError_t mvp_whole_launch(Ctx& c, const PointsDev& P, const float* Q, float shift, float* Y, cudaStream_t st) {
+  // (a loaded tuning file: the key holds the block counts, so they were read)
+  TuneScope scope(c, c.tune_cache.empty() ? 1.0 : tuned_scale(c, tune_key(c, "mvp", P, P, 1, KRR_FP32)));
+  const Plan pl = f32_plan(c, P, P);
+  const size_t ctas = (size_t)((P.nblk + NW - 1) / NW);
+  void *part, *fac, *tick;
+  cudaError_t e;
+  if ((e = c.ws.get("mvp.part", sizeof(double) * pl.splits * (size_t)P.Npad, &part))) return e;
+  if ((e = c.ws.get("mvp.fac", sizeof(float) * (size_t)P.Npad, &fac))) return e;
+  const bool fresh = c.ws.slots.find("mvp.tick") == c.ws.slots.end();
+  constexpr size_t TICKS = WHOLE_MAX_N / 32 / NW + 1;
+  if (ctas > TICKS) return cudaErrorNotSupported;
+  if ((e = c.ws.get("mvp.tick", sizeof(unsigned) * TICKS, &tick))) return e;
+  if (fresh && (e = cudaMemsetAsync(tick, 0, sizeof(unsigned) * TICKS, st))) return e;
+  MvpParams p{};
+  p.xt = P.xs;
+  p.Nt = P.N;
+  p.Nt_pad = P.Npad;
+  p.tctr = P.ctr;
+  p.torder = P.order;
+  p.tn_exp = P.n_exp;
+  p.nblk = P.nblk;
+  p.xs = P.xs;
+  p.ntiles = source_tiles(P);
+  p.s = P.scale;
+  p.part_stride = P.Npad;
+  p.err = c.d_err;
+  p.row_lo = c.row_lo;
+  p.row_hi = c.row_hi;
+  p.part = (double*)part;
+  p.fac = (float*)fac;
+  p.q_orig = Q;
+  p.perm = P.perm;
+  p.tick = (unsigned*)tick;
+  p.y_orig = Y;
+  p.shift = shift;
+  p.pdl = P.counts_read;
+  return f32_any(p, P.d, P.kfam, P.T, pl, st, true);
 }
 
 cudaError_t mvp_multi_reserve(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, int m,

@@ -629,7 +629,7 @@ cudaError_t scatter_orig(const float* in, int64_t Npad, int64_t N, int m, const 
 }
 
 cudaError_t prepare_points(Ctx& c, const float* X, int64_t N, int d, float sigma,
-                           const char* tag, PointsDev& P, cudaStream_t st) {
+                           const char* tag, PointsDev& P, cudaStream_t st, bool read_counts) {
   const std::string t(tag);
   const int d_in = d;
   d = padded_dim(d_in);
@@ -738,6 +738,8 @@ cudaError_t prepare_points(Ctx& c, const float* X, int64_t N, int d, float sigma
                                            OrderArgs{P.sb_flag, P.nsb, P.sb_order, P.sb_nexp, hc ? hc + 1 : nullptr});
   count_launch();
   if ((e = cudaGetLastError())) return e;
+  P.counts_read = read_counts;
+  if (!read_counts) return cudaSuccess;
   if (!hc) {
     if ((e = cudaMemcpyAsync(&counts[0], P.n_exp, sizeof(int), cudaMemcpyDeviceToHost, st))) return e;
     if ((e = cudaMemcpyAsync(&counts[1], P.sb_nexp, sizeof(int), cudaMemcpyDeviceToHost, st))) return e;
