@@ -393,6 +393,48 @@ __global__ void store_z_kernel(KState* S0, const float* __restrict__ z, float* _
   KRR_GRID_LOOP(i) zj[i] = z[co + i];
 }
 
+// After both passes (S->h1, S->h2, S->wnorm2 = |w|^2): the Hessenberg column,
+// the Givens update of Alg. 1's least squares problem and the continuation
+// test.  One thread.
+__device__ void givens_step(KState* S, int j) {
+  const int nj = j + 1;
+  // |w - V h2|^2 = |w|^2 - |h2|^2 (V orthonormal)
+  double hh = 0.0;
+  for (int c = 0; c < nj; ++c) hh += S->h2[c] * S->h2[c];
+  const double wn2 = fmax(S->wnorm2 - hh, 0.0);
+  double* Hj = S->H + (int64_t)j * (MMAX + 1);
+  for (int c = 0; c < nj; ++c) Hj[c] = S->h1[c] + S->h2[c];
+  const double hnext = sqrt(wn2);
+  Hj[nj] = hnext;
+  // apply the previous rotations to the new column, then a new rotation that
+  // zeroes H[j+1, j]
+  for (int c = 0; c < j; ++c) {
+    const double t0 = S->cs[c] * Hj[c] + S->sn[c] * Hj[c + 1];
+    const double t1 = -S->sn[c] * Hj[c] + S->cs[c] * Hj[c + 1];
+    Hj[c] = t0;
+    Hj[c + 1] = t1;
+  }
+  const double a = Hj[j], b = Hj[j + 1];
+  const double rr = hypot(a, b);
+  const double cj = rr > 0.0 ? a / rr : 1.0, sj = rr > 0.0 ? b / rr : 0.0;
+  S->cs[j] = cj;
+  S->sn[j] = sj;
+  Hj[j] = rr;
+  Hj[j + 1] = 0.0;
+  const double gj = S->g[j];
+  S->g[j] = cj * gj;
+  S->g[j + 1] = -sj * gj;
+  S->relres_est = fabs(S->g[j + 1]) / S->bnorm;
+  S->outer_total += 1;
+  S->kcols = j + 1;
+  // lucky breakdown: w lies in the span of V, the least-squares residual is exact
+  const bool lucky = !(hnext > 1e-14 * rr) || !isfinite(hnext);
+  S->lucky = lucky ? 1 : 0;
+  S->wnorm2 = hnext;  // reused by cgs_final as the normaliser
+  const bool more = !lucky && (j + 1 < S->m) && S->relres_est > S->tol_cycle;
+  S->arn_cont = more ? 1 : 0;
+}
+
 // h1[i] = (w, v_i), i = 0..j  (first Gram-Schmidt pass).
 __global__ void cgs_dots_kernel(KState* S0, const double* __restrict__ V, int64_t vstride,
                                 const double* __restrict__ w, int64_t Np, double* partials,
@@ -476,41 +518,7 @@ __global__ void cgs_update_kernel(KState* S0, const double* __restrict__ V, int6
   }
   if (threadIdx.x != 0) return;
   S->ticket = 0u;
-  // |w - V h2|^2 = |w|^2 - |h2|^2 (V orthonormal)
-  double hh = 0.0;
-  for (int c = 0; c < nj; ++c) hh += S->h2[c] * S->h2[c];
-  const double wn2 = fmax(S->wnorm2 - hh, 0.0);
-  double* Hj = S->H + (int64_t)j * (MMAX + 1);
-  for (int c = 0; c < nj; ++c) Hj[c] = S->h1[c] + S->h2[c];
-  const double hnext = sqrt(wn2);
-  Hj[nj] = hnext;
-  // apply the previous rotations to the new column, then a new rotation that
-  // zeroes H[j+1, j]
-  for (int c = 0; c < j; ++c) {
-    const double t0 = S->cs[c] * Hj[c] + S->sn[c] * Hj[c + 1];
-    const double t1 = -S->sn[c] * Hj[c] + S->cs[c] * Hj[c + 1];
-    Hj[c] = t0;
-    Hj[c + 1] = t1;
-  }
-  const double a = Hj[j], b = Hj[j + 1];
-  const double rr = hypot(a, b);
-  const double cj = rr > 0.0 ? a / rr : 1.0, sj = rr > 0.0 ? b / rr : 0.0;
-  S->cs[j] = cj;
-  S->sn[j] = sj;
-  Hj[j] = rr;
-  Hj[j + 1] = 0.0;
-  const double gj = S->g[j];
-  S->g[j] = cj * gj;
-  S->g[j + 1] = -sj * gj;
-  S->relres_est = fabs(S->g[j + 1]) / S->bnorm;
-  S->outer_total += 1;
-  S->kcols = j + 1;
-  // lucky breakdown: w lies in the span of V, the least-squares residual is exact
-  const bool lucky = !(hnext > 1e-14 * rr) || !isfinite(hnext);
-  S->lucky = lucky ? 1 : 0;
-  S->wnorm2 = hnext;  // reused by cgs_final as the normaliser
-  const bool more = !lucky && (j + 1 < S->m) && S->relres_est > S->tol_cycle;
-  S->arn_cont = more ? 1 : 0;
+  givens_step(S, j);
 }
 
 // v_{j+1} = (w - V h2) / h_{j+1,j}
@@ -532,6 +540,110 @@ __global__ void cgs_final_kernel(KState* S0, double* __restrict__ V, int64_t vst
     for (int c = 0; c < nj; ++c) wi -= h2s[c] * V[(int64_t)c * Np + i];
     vn[i] = wi * inv;
   }
+}
+
+// ---- both Gram-Schmidt passes, the Givens step and v_{j+1} in one launch for
+// Np <= STEP_MAX_NP: one cluster per column, a thread keeps its R rows of w in
+// registers.  A warp sums one basis vector at a time over its CTA's rows of w
+// in shared memory (8 R FP64 operations per lane and 5 for the warp, against
+// a block sum per vector in the kernels above), and the CTAs exchange their
+// sums through distributed shared memory.  The three kernels took 34, 47 and
+// 5 us at 2,000 points and 15 vectors.
+template <int R>
+__global__ void __launch_bounds__(STEP_T)
+    cgs_cluster_kernel(KState* S0, double* __restrict__ V, int64_t vstride, const double* __restrict__ w, int64_t Np,
+                       int pred) {
+  __shared__ double ws[R * STEP_T];                  // this CTA's rows of w
+  __shared__ double part[2][STEP_CL][MMAX + 2];      // per pass: every CTA's sums
+  __shared__ double h[MMAX + 2], inv_s;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, rank = blockIdx.x, col = blockIdx.y;
+  KState* S = S0 + col;
+  if (!col_flag(S, pred)) return;  // uniform over the cluster
+  cluster_arrive();                // every CTA has started: awaited before the first exchange
+  const int j = S->j, nj = j + 1;
+  V += (int64_t)col * vstride;
+  w += (int64_t)col * Np;
+  double wr[R];
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    const int64_t i = (int64_t)(k * STEP_CL + rank) * STEP_T + t;
+    wr[k] = i < Np ? w[i] : 0.0;
+    ws[k * STEP_T + t] = wr[k];
+  }
+  __syncthreads();
+  // sums over the cluster of v_c w for c < nj (and |w|^2 as number nj when
+  // norm is set) into h
+  auto dots = [&](int pass, bool norm) {
+    for (int c = warp; c < nj + (norm ? 1 : 0); c += STEP_T / 32) {
+      const double* vc = V + (int64_t)c * Np;
+      double a = 0.0;
+#pragma unroll
+      for (int k = 0; k < R; ++k) {
+        const int64_t i0 = (int64_t)(k * STEP_CL + rank) * STEP_T;
+        if (i0 >= Np) break;  // Np is a multiple of STEP_T
+        double u[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const double x = ws[k * STEP_T + 32 * e + lane];
+          u[e] = (c < nj ? vc[i0 + 32 * e + lane] : x) * x;
+        }
+        a += tree8(u);
+      }
+      a = warp_sum(a);
+      if (pass == 0 && c == warp) cluster_wait();  // (each warp's first)
+      if (lane < STEP_CL) {
+        uint32_t d;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(smem_addr(&part[pass][rank][c])), "r"(lane));
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(d), "d"(a) : "memory");
+      }
+    }
+    if (pass == 0 && warp >= nj) cluster_wait();  // warps without a vector
+    cluster_arrive();
+    cluster_wait();
+    if (t < nj + (norm ? 1 : 0)) {
+      double u[STEP_CL];
+#pragma unroll
+      for (int r = 0; r < STEP_CL; ++r) u[r] = part[pass][r][t];
+      h[t] = tree8(u);
+    }
+    __syncthreads();
+  };
+  dots(0, false);
+  if (rank == 0 && t < nj) S->h1[t] = h[t];
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    const int64_t i = (int64_t)(k * STEP_CL + rank) * STEP_T + t;
+    if (i < Np)
+      for (int c = 0; c < nj; ++c) wr[k] -= h[c] * V[(int64_t)c * Np + i];
+    ws[k * STEP_T + t] = wr[k];
+  }
+  __syncthreads();
+  dots(1, true);
+  // v_{j+1} = (w - V h2) / h_{j+1,j}, every CTA with the same norm; a breakdown
+  // leaves the next vector unused
+  if (t == 0) {
+    double hh = 0.0;
+    for (int c = 0; c < nj; ++c) hh += h[c] * h[c];
+    const double hnext = sqrt(fmax(h[nj] - hh, 0.0));
+    inv_s = hnext > 0.0 && isfinite(hnext) ? 1.0 / hnext : 0.0;
+  }
+  __syncthreads();
+  const double inv = inv_s;
+  if (inv > 0.0) {
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      const int64_t i = (int64_t)(k * STEP_CL + rank) * STEP_T + t;
+      if (i >= Np) continue;
+      for (int c = 0; c < nj; ++c) wr[k] -= h[c] * V[(int64_t)c * Np + i];
+      V[(int64_t)nj * Np + i] = wr[k] * inv;
+    }
+  }
+  // the state: rank 0, after its rows (S->j was read by all before the exchanges)
+  if (rank != 0) return;
+  if (t < nj) S->h2[t] = h[t];
+  if (t == 0) S->wnorm2 = h[nj];
+  __syncthreads();
+  if (t == 0) givens_step(S, j);
 }
 
 // One thread per column: advance the columns whose Arnoldi process
@@ -979,27 +1091,39 @@ struct Solver {
     return e;
   }
 
-  // The rest of a CG step from the product's partial sums (MvpOut::finish)
-  static cudaError_t cg_step(void* arg, const ProdSums& sums, cudaStream_t st) {
-    Solver& s = *(Solver*)arg;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(STEP_CL, (unsigned)s.mc);
+  // Launch configuration of the cluster kernels (one cluster per column), and
+  // their instance for this many rows per thread.  at[0] is the cluster size.
+  void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at) const {
+    cfg.gridDim = dim3(STEP_CL, (unsigned)mc);
     cfg.blockDim = dim3(STEP_T);
     cfg.stream = st;
-    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = STEP_CL;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+  }
+  template <typename F>
+  F rows_of(F k1, F k2, F k4, F k8) const {
+    const int64_t rows = (Np + STEP_CL * STEP_T - 1) / (STEP_CL * STEP_T);
+    return rows <= 1 ? k1 : rows <= 2 ? k2 : rows <= 4 ? k4 : k8;
+  }
+
+  // The rest of a CG step from the product's partial sums (MvpOut::finish)
+  static cudaError_t cg_step(void* arg, const ProdSums& sums, cudaStream_t st) {
+    Solver& s = *(Solver*)arg;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[2];
+    s.cluster_config(cfg, at);
+    cfg.stream = st;
     // (a product of several columns or in 16 bits may end in a join of streams)
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = s.mc == 1 && s.inner_prec == KRR_FP32 ? 2 : 1;
-    const int64_t rows = (s.Np + STEP_CL * STEP_T - 1) / (STEP_CL * STEP_T);  // per thread
-    auto* kernel = rows <= 1 ? cg_step_kernel<1> : rows <= 2 ? cg_step_kernel<2>
-                   : rows <= 4 ? cg_step_kernel<4> : cg_step_kernel<8>;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, s.S, sums, s.z, s.rr, s.p, s.G, s.cg_c);
+    if (s.mc == 1 && s.inner_prec == KRR_FP32) cfg.numAttrs = 2;
+    cudaError_t e = cudaLaunchKernelEx(
+        &cfg, s.rows_of(cg_step_kernel<1>, cg_step_kernel<2>, cg_step_kernel<4>, cg_step_kernel<8>), s.S, sums, s.z,
+        s.rr, s.p, s.G, s.cg_c);
     count_launch();
     return e;
   }
@@ -1044,9 +1168,19 @@ struct Solver {
     cols.state_stride = sizeof(KState);
     cudaError_t e = mvp_acc_launch(c, P, z, zero, gamma, 0.0, nullptr, 1.0, w, nullptr, st, cols);
     if (e) return e;
-    cgs_dots_kernel<<<vgrid(), VT, 0, st>>>(S, V, vstride(), w, Np, partials, PRED_STEP); count_launch();
-    cgs_update_kernel<<<vgrid(), VT, 0, st>>>(S, V, vstride(), w, Np, partials, PRED_STEP); count_launch();
-    cgs_final_kernel<<<vgrid(), VT, 0, st>>>(S, V, vstride(), w, Np, PRED_STEP); count_launch();
+    if (Np <= STEP_MAX_NP) {
+      cudaLaunchConfig_t cfg = {};
+      cudaLaunchAttribute at[1];
+      cluster_config(cfg, at);
+      e = cudaLaunchKernelEx(&cfg, rows_of(cgs_cluster_kernel<1>, cgs_cluster_kernel<2>, cgs_cluster_kernel<4>,
+                                           cgs_cluster_kernel<8>), S, V, vstride(), (const double*)w, Np, (int)PRED_STEP);
+      count_launch();
+      if (e) return e;
+    } else {
+      cgs_dots_kernel<<<vgrid(), VT, 0, st>>>(S, V, vstride(), w, Np, partials, PRED_STEP); count_launch();
+      cgs_update_kernel<<<vgrid(), VT, 0, st>>>(S, V, vstride(), w, Np, partials, PRED_STEP); count_launch();
+      cgs_final_kernel<<<vgrid(), VT, 0, st>>>(S, V, vstride(), w, Np, PRED_STEP); count_launch();
+    }
     arn_advance_kernel<<<1, 32, 0, st>>>(S, mc, G, arn_c); count_launch();
     return cudaGetLastError();
   }

@@ -61,6 +61,7 @@ struct AccParams {
   const float* ql;   // source weights lo
   const float* tbox; // source tile boxes
   int ntiles, tiles_per_split;
+  int sub;  // parts of a tile that are splits of their own (tiles_per_split 1), else 1
   double* part;      // [columns][splits][Npad]
   int splits;
   int* err;
@@ -227,7 +228,8 @@ __global__ void __launch_bounds__(NT) mvp_acc_kernel(const AccParams p) {
     }
   }
 
-  const int t_begin = blockIdx.y * p.tiles_per_split;
+  const int t_begin = (int)blockIdx.y / p.sub * p.tiles_per_split;
+  const int j0 = (int)blockIdx.y % p.sub * (TS / p.sub), j1 = j0 + TS / p.sub;
   const int nt = min(p.ntiles, t_begin + p.tiles_per_split) - t_begin;
   float S[TA], L[TA];
 #pragma unroll
@@ -279,14 +281,14 @@ __global__ void __launch_bounds__(NT) mvp_acc_kernel(const AccParams p) {
       }
       if (s2h * dist2 <= far_e<KF>()) {
 #pragma unroll 2
-        for (int j = 0; j < TS; ++j) {
+        for (int j = j0; j < j1; ++j) {
           const float qh = sq[j], ql = sl[j];
 #pragma unroll
           for (int u = 0; u < TA; ++u)
             acc_pair<D, KF>(xi[u], st + j, qh, ql, S[u], L[u], p.k, tab_h, tab_l);
         }
       } else {
-        for (int j = 0; j < TS; ++j) {
+        for (int j = j0; j < j1; ++j) {
           const float qh = sq[j];
 #pragma unroll
           for (int u = 0; u < TA; ++u) {
@@ -380,7 +382,8 @@ __global__ void __launch_bounds__(NT, (D > 8 ? 1 : 2)) mvp_accm_kernel(const Acc
     }
   }
 
-  const int t_begin = blockIdx.y * p.tiles_per_split;
+  const int t_begin = (int)blockIdx.y / p.sub * p.tiles_per_split;
+  const int j0 = (int)blockIdx.y % p.sub * (TS / p.sub), j1 = j0 + TS / p.sub;
   const int nt = min(p.ntiles, t_begin + p.tiles_per_split) - t_begin;
   float S[AM], L[AM];
 #pragma unroll
@@ -434,7 +437,7 @@ __global__ void __launch_bounds__(NT, (D > 8 ? 1 : 2)) mvp_accm_kernel(const Acc
       }
       if (s2h * dist2 <= far_e<KF>()) {
 #pragma unroll 1
-        for (int j = 0; j < TS; ++j) {
+        for (int j = j0; j < j1; ++j) {
           float H, L2;
           acc_kval<D, KF>(xi, st + j, p.k, tab_h, tab_l, H, L2);
 #pragma unroll
@@ -443,7 +446,7 @@ __global__ void __launch_bounds__(NT, (D > 8 ? 1 : 2)) mvp_accm_kernel(const Acc
         }
       } else {
 #pragma unroll 1
-        for (int j = 0; j < TS; ++j) {
+        for (int j = j0; j < j1; ++j) {
           float r2 = 0.f;
 #pragma unroll
           for (int k = 0; k < D; ++k) {
@@ -640,11 +643,11 @@ cudaError_t launch_any(const AccParams& p, int d, int kf, int splits, int ncols,
 }
 
 struct AccPlan {
-  int splits, tiles_per_split;
+  int splits, tiles_per_split, sub;
 };
 
 // scale: the autotuner's factor on the modelled split count (1: the model).
-AccPlan acc_plan(const PointsDev& P, int num_sms, int plan_slots, int ncols, double scale) {
+AccPlan acc_plan(const PointsDev& P, int num_sms, int plan_slots, int ncols, double scale, bool parts) {
   const int ntiles = source_tiles(P);
   // one target per thread in the multi-column kernel, ACC_TA otherwise
   const int ta = (ncols > 1 || P.d > 8) ? 1 : ACC_TA;
@@ -656,6 +659,15 @@ AccPlan acc_plan(const PointsDev& P, int num_sms, int plan_slots, int ncols, dou
   AccPlan pl;
   pl.tiles_per_split = (ntiles + splits - 1) / splits;
   pl.splits = (ntiles + pl.tiles_per_split - 1) / pl.tiles_per_split;
+  // one tile per split and still fewer CTAs than SMs: halves or quarters of a
+  // tile (2,000 points: one column 54 us with whole tiles and 16 with parts, 11
+  // columns 175 and 91).  Not in krr_mll_grad, whose results keep their bits.
+  pl.sub = 1;
+  if (parts && scale == 1.0 && pl.tiles_per_split == 1)
+    while (pl.sub < 4 && ctas * pl.splits * 2 <= (plan_slots > 0 ? plan_slots : num_sms)) {
+      pl.sub *= 2;
+      pl.splits *= 2;
+    }
   return pl;
 }
 
@@ -685,7 +697,7 @@ cudaError_t autotune_acc(Ctx& c, const PointsDev& P, int ncols, cudaStream_t st,
   for (double s : TUNE_SCALES) {
     c.tune_cache[key] = s;
     if (s > 1.0 &&
-        8.0 * acc_plan(P, c.num_sms, c.plan_slots, ncols, s).splits * ncols * (double)P.Npad > TUNE_MAX_BYTES)
+        8.0 * acc_plan(P, c.num_sms, c.plan_slots, ncols, s, !c.morton).splits * ncols * (double)P.Npad > TUNE_MAX_BYTES)
       continue;
     auto run = [&]() {
       return mvp_acc_launch(c, P, (const float*)qv, (const float*)qv, 0.f, 0.0, nullptr, 1.0, (double*)yv,
@@ -725,7 +737,7 @@ cudaError_t mvp_acc_reserve(Ctx& c, const PointsDev& P, cudaStream_t st, int nco
     if (te) return te;
   }
   TuneScope scope(c, tuned_scale(c, key));
-  const AccPlan pl = acc_plan(P, c.num_sms, c.plan_slots, ncols, c.split_scale);
+  const AccPlan pl = acc_plan(P, c.num_sms, c.plan_slots, ncols, c.split_scale, !c.morton);
   void* v;
   cudaError_t e;
   if ((e = c.ws.get("acc.part", sizeof(double) * ncols * pl.splits * (size_t)P.Npad, &v))) return e;
@@ -768,9 +780,10 @@ cudaError_t mvp_acc_launch(Ctx& c, const PointsDev& P, const float* qh, const fl
   const double sd = std::sqrt(P.s2);
   p.k.sh = (float)sd;
   p.k.sl = (float)(sd - (double)p.k.sh);
-  const AccPlan pl = acc_plan(P, c.num_sms, c.plan_slots, ncols, c.split_scale);
+  const AccPlan pl = acc_plan(P, c.num_sms, c.plan_slots, ncols, c.split_scale, !c.morton);
   p.tiles_per_split = pl.tiles_per_split;
   p.splits = pl.splits;
+  p.sub = pl.sub;
   p.active = cols.active;
   p.state_stride = cols.state_stride;
   void *part, *dpart, *dcnt;
