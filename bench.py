@@ -481,6 +481,8 @@ def run_libkrr(args):
                 "unit": "Gpairs/s", "frac": achieved * 1e9 / peak_pairs,
                 "traffic": traffic_bytes(tensor_exp),
                 "kernel": kernel_name, "launch_ms": kern_ms,
+                "pairs": "all N^2; the kernel leaves out source tiles whose kernel values "
+                         "are exact zeros in its arithmetic (the sums are the same bit for bit)",
                 "peak_source": "measured on this GPU: min(MUFU.EX2 rate, FP32 lane rate / FP32 "
                                f"operations per pair) = min({ex2_rate / 1e12:.2f}e12, "
                                f"{fp32_lanes / 1e12:.2f}e12/{fp32_per_pair})",
@@ -778,11 +780,12 @@ def matern_form(K, torch, inputs, X, q, rank, dev, stream, ex2_rate, fp32_lanes)
     n = X.shape[0]
     pairs = float(n) * n
     kern_ms = prof["product_ms"] / max(prof["product_launches"], 1)
-    # direct form per pair: d differences, d multiply-adds, three multiplies
-    # (r = r^2 rsqrt(r^2), a = s r, the exponent), the (1 + a) e FMA and the
-    # weighted accumulate on the FP32 lanes; one rsqrt and one EX2 on MUFU
+    # direct form per pair: d differences, d multiply-adds, two multiplies
+    # (a = s r, the exponent), the (1 + a) e FMA and the weighted accumulate on
+    # the FP32 lanes; one square root (at the reciprocal's rate) and one EX2 on
+    # MUFU
     d = X.shape[1]
-    fp32_ops = 2 * d + 5
+    fp32_ops = 2 * d + 4
     peak = min(fp32_lanes / fp32_ops, 1.0 / (1.0 / ex2_rate + 1.0 / rsqrt_rate))
     product = {"N": n, "d": d, "h": hl, "step_ms": ms / reps, "kernel_ms": kern_ms,
                "Gpairs_per_s": pairs / (kern_ms / 1e3) / 1e9,
