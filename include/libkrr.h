@@ -149,8 +149,9 @@ typedef enum {
      *     once per product shape when they reserve it (a few products,
      *     before any graph capture) and keep the faster.
      * Same results to the float32 bar (and the reduced-precision bars).  On
-     * GB300, 16 columns at 2^20 points: float32 370 / 434 / 552 ms, f16
-     * 260 / 261 / 378 ms for 1 / 0 / 2.  Other values: KRR_ERR_INVALID_ARG. */
+     * GB300, 16 columns at 2^20 points in float32: 65 / 84 / 546 ms for
+     * 1 / 0 / 2 (2 visits every tile of pairs).  Other values:
+     * KRR_ERR_INVALID_ARG. */
     KRR_OPT_TCGEN05 = 1,
     /* value: a krr_kernel_family.  The kernel function every product and
      * solver of this handle uses (default KRR_KERNEL_GAUSSIAN).  Under
@@ -237,7 +238,8 @@ krr_status krr_set_option(krr_handle h, int option, int value);
  * The call may wait briefly for the point preparation (Hilbert sort and block
  * metadata) to read the block counts that size the product grids (single
  * columns in float32 of up to 16384 points up to 8 dimensions do not need
- * them); the product itself is asynchronous on device arrays. */
+ * them); the product itself is asynchronous on device arrays, which must stay
+ * valid until it is complete. */
 krr_status krr_kernel_mvp(krr_handle h, const float* X, int64_t N, int d,
                           float sigma, float gamma, const float* Q, int m,
                           float* Y, krr_precision prec, void* stream);
@@ -383,9 +385,10 @@ krr_status krr_mll_grad(krr_handle h, const float* X, int64_t N, int d,
  * the result).  Outputs are HOST doubles; any may be NULL. */
 krr_status krr_measure_alu_peaks(krr_handle h, double* ex2_per_s, double* ffma_per_s,
                                  double* ffma2_lanes_per_s, void* stream);
-/* Reciprocal square roots (rsqrtf, the one the Matern kernel takes per pair)
- * per second on the handle's device at its current clocks, measured the same
- * way (a few ms of GPU time; waits).  rsqrt_per_s: HOST double, not NULL. */
+/* Reciprocal square roots (rsqrtf; the Matern kernel takes one square root per
+ * pair on the same unit) per second on the handle's device at its current
+ * clocks, measured the same way (a few ms of GPU time; waits).  rsqrt_per_s:
+ * HOST double, not NULL. */
 krr_status krr_measure_rsqrt_rate(krr_handle h, double* rsqrt_per_s, void* stream);
 
 /* Rates behind the reduced-precision design, measured the same way (a few

@@ -79,6 +79,11 @@ struct PointsDev {
 // Targets per super-block.
 constexpr int SB = 256;
 
+// Source tiles one CTA can list as contributing (live_tiles in mvp_tc.cu);
+// longer ranges are walked whole.  One bit each: twice as many would take the
+// shared memory that lets two CTAs of the d = 8 tcgen05 kernel share an SM.
+constexpr int LIVE_TILES = 4096;
+
 // Source tiles (of SB points) that hold points.  The prepared arrays are padded
 // to PAD = 8 tiles; the tiles behind the last point have zero weights and are
 // left out of every product (4,097 points: 17 tiles of 24).

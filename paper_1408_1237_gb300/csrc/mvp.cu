@@ -634,10 +634,12 @@ cudaError_t launch_typed(const MvpParams& p, int splits, cudaStream_t st) {
 
 // Split count minimising the makespan ceil(blocks*S/slots) * (ceil(tiles/S) +
 // setup), setup = a CTA's fixed cost in units of one source tile.
+// No split is longer than LIVE_TILES where 64 splits allow it.
 int choose_splits(int64_t blocks, int tiles, int slots, double setup = 0.0) {
-  int best = 1;
+  const int least = std::min((tiles + LIVE_TILES - 1) / LIVE_TILES, 64);
+  int best = least;
   double best_cost = 1e300;
-  for (int s = 1; s <= std::min(tiles, 64); ++s) {
+  for (int s = least; s <= std::min(tiles, 64); ++s) {
     const double waves = std::ceil((double)blocks * s / slots);
     const double cost = waves * (std::ceil((double)tiles / s) + setup);
     if (cost < best_cost - 1e-9) {

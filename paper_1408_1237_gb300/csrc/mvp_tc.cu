@@ -91,7 +91,7 @@ struct TcParams {
 // that is not finite compares as near).  The gaps are shortened by a few units
 // in the last place of the coordinates, since the boxes are rounded.
 constexpr float CUT_F32 = 128.f, CUT_F16 = 26.f;
-constexpr int LIVE_WORDS = 256;  // 8192 tiles per CTA; longer ranges keep every tile
+constexpr int LIVE_WORDS = LIVE_TILES / 32;
 
 // Writes bit r of mask for every live tile t_begin + r, r < nt, and returns
 // their number; blk: the CTA's super-block.  All threads call it.

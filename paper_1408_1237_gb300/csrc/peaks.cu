@@ -1,7 +1,8 @@
 // Issue-rate microbenchmarks for the ALU roofline of the kernel product:
 // MUFU.EX2 (ex2.approx.ftz.f32), scalar FFMA and packed FFMA2 (f32x2)
 // results per second on this GPU, measured at its current clocks; the
-// reciprocal square root (rsqrtf) the Matern kernel takes per pair; and the
+// reciprocal square root (rsqrtf; the Matern kernel takes a square root per
+// pair on the same unit); and the
 // rates that decide the reduced-precision design: packed half-precision
 // exponentials (ex2.approx.f16x2, ex2.approx.ftz.bf16x2: two values per
 // instruction) and the warp-level tensor-core MMA (mma.sync m16n8k16, f16 in,
