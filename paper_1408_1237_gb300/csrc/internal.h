@@ -327,9 +327,9 @@ struct MvpOut {
   // not cancel (gather_sorted; null: none does, as in the solvers, whose
   // iteration stops on a product that is not finite wherever it appears)
   const int* qbad = nullptr;
-  // an inner product of a solver's preconditioner, which tolerates rounding:
-  // several columns take the tensor-core kernels' less exact form
-  bool inner = false;
+  // several columns take the tensor-core kernels' form that is as exact as the
+  // single-column kernels (the prediction product, in whose place it stands)
+  bool fine = false;
   // y = alpha * (K_hat q + shift q) + beta * u, sorted order
   float alpha = 1.f, beta = 0.f;
   const float* u = nullptr;
@@ -373,8 +373,7 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& T, const PointsDev& S, con
                              const float* qdiag, float shift, krr_precision prec, const MvpOut& o,
                              cudaStream_t st);
 // ---- mvp_tc.cu: tensor-core partial sums of the expanded-form warp blocks
-// fine = false: the form for the inner products of a solver's preconditioner
-// (KRR_FP32 only; see the kernel).
+// fine: the more exact form (KRR_FP32 only; see the kernel).
 // dry = true only sets the kernel attributes (before any graph capture).
 cudaError_t mvp_tc_partials(Ctx& c, const PointsDev& T, const PointsDev& S, const float* Q, int m,
                             krr_precision prec, bool fine, int splits, int tiles_per_split, double* part,

@@ -685,6 +685,7 @@ krr_status krr_kernel_mvp_rect(krr_handle h, const float* Xt, int64_t Nt, const 
       o.qbad = (const int*)qbad;
       o.perm = T.perm;
       o.out_orig = dY + (size_t)col * Nt;
+      o.fine = true;
       e = mc == 1 ? mvp_launch(c, T, S, qc, nullptr, 0.f, prec, o, st)
                   : mvp_multi_launch(c, T, S, qc, mc, nullptr, 0.f, prec, o, st);
       if (e) return cuda_error(c, e, fn);

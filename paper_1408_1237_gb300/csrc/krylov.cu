@@ -1132,7 +1132,6 @@ struct Solver {
   // for every column whose CG continues
   cudaError_t cg_iteration() {
     MvpOut o;
-    o.inner = true;
     if (Np <= STEP_MAX_NP) {
       o.active = &G->cg_any;
       o.finish = cg_step;

@@ -940,7 +940,6 @@ cudaError_t autotune_mvp(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, int m
   }
   MvpOut o;
   o.out_f = (float*)yv;
-  o.inner = tcgen05_only;  // a solver's choice
   const bool single = m == 1 && prec == KRR_FP32;
   auto run = [&]() {
     return single ? mvp_launch(c, Tp, Sp, (const float*)qv, nullptr, 0.f, prec, o, st)
@@ -1466,7 +1465,7 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, c
     e = tc5_on(c, prec, m, Tp)
             ? mvp_umma_partials(c, Tp, Sp, Q, m, prec == KRR_FP32, prec == KRR_BF16, pt.splits,
                                 pt.tiles_per_split, (double*)part, p.fac, o.active, o.qbad, st)
-            : mvp_tc_partials(c, Tp, Sp, Q, m, prec, !o.inner, pt.splits, pt.tiles_per_split, (double*)part,
+            : mvp_tc_partials(c, Tp, Sp, Q, m, prec, o.fine, pt.splits, pt.tiles_per_split, (double*)part,
                               p.fac, o.active, o.qbad, st);
     if (e) return e;
   }
@@ -1482,7 +1481,7 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, c
     }
     if (use_dirtc(c, Tp)) {
       if ((e = mvp_dirtc_partials(c, Tp, Sp, Q, m, prec, pd.splits, pd.tiles_per_split, nexp, p.tn_exp,
-                                  (double*)partd, p.fac, o.active, !o.inner, dst, false)))
+                                  (double*)partd, p.fac, o.active, o.fine, dst, false)))
         return e;
     } else if ((e = dirm_dispatch(p, Tp.d, Tp.kfam, Q, Sp.Npad, m, SB / 32, nexp, pd, dst, true))) {
       return e;

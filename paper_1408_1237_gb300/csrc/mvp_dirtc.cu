@@ -18,10 +18,10 @@
 //     below 3 * 2^-20.  No format conversion is needed (tf32 is float32's
 //     layout), and tf32 has float32's exponent range, so small kernel values
 //     and large weights keep their precision.  Two forms (SPLIT):
-//      1: Ph = P with its low bits cleared, one accumulator for all three.  For
-//         the inner products of the solvers' preconditioner.  Relative error
-//         of a product 1.8e-6 (20,011 points, d = 3) to 2.5e-6 (16,385, d = 8);
-//      2: for every other product.  Ph is rounded, which gives the low parts
+//      1: Ph = P with its low bits cleared, one accumulator for all three.
+//         Relative error of a product 1.8e-6 (20,011 points, d = 3) to 2.5e-6 (16,385, d = 8);
+//      2: where it takes the place of single-column products (prediction of
+//         several columns).  Ph is rounded, which gives the low parts
 //         both signs, so that what the split drops does not add up; the tensor
 //         cores truncate when they accumulate, so Ph Qh goes into fresh
 //         accumulators every FOLD sources, folded in float32, and the two small

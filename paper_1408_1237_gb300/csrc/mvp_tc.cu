@@ -238,12 +238,12 @@ __device__ __forceinline__ float kv_value(const float (&h)[D + 1], const float (
   return v;
 }
 
-// SPLIT: 0 single operands; 1 hi + lo, for the inner products of the solvers'
-// preconditioner; 2 hi + lo with Ph Qh in fresh accumulators every FOLD sources
-// (the tensor cores truncate when they accumulate) and the small products in
-// accumulators of their own, for every other float32 product.  Relative error
-// at 131,072 points in the cube 1.5e-6 with 1 and 2.8e-7 with 2, as the
-// single-column kernels (2.5e-7), for 2 to 5% more time.
+// SPLIT: 0 single operands; 1 hi + lo; 2 hi + lo with Ph Qh in fresh
+// accumulators every FOLD sources (the tensor cores truncate when they
+// accumulate) and the small products in accumulators of their own, where it
+// takes the place of single-column products.  Relative error at 131,072 points
+// in the cube 1.5e-6 with 1 and 2.8e-7 with 2 (2.5e-7 for the single-column
+// kernels), for 5 to 9% more time.
 template <int D, int MT, int NRT, int SPLIT, bool BF>
 __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
   using L = ExpLayout<D>;
