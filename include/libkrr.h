@@ -181,8 +181,9 @@ typedef enum {
     /* Target-row shard emulation (the row partition a multi-GPU product
      * would use, run on one GPU): with SHARD_COUNT = P > 1, krr_kernel_mvp
      * on this handle computes and writes only shard SHARD_INDEX = k of its
-     * target rows: the sorted (Hilbert-order) super-blocks
-     * [k nsb / P, (k+1) nsb / P) of 256 targets, that is 1/P of the work.
+     * target rows: the sorted super-blocks (Hilbert order; in 16 bits see
+     * krr_kernel_mvp) [k nsb / P, (k+1) nsb / P) of 256 targets, that is 1/P
+     * of the work.
      * The other rows of Y are left as they were (a host Y is uploaded
      * first).  The plans are those of the whole product, so the P shards
      * written into one Y equal the unsharded product bit for bit.  Other
@@ -234,7 +235,10 @@ krr_status krr_set_option(krr_handle h, int option, int value);
  * (tensor cores for compact target blocks).
  * prec: KRR_FP32 (max relative error per element, against the FP64 sum
  * scaled by sum_j |Q_jc| K_hat_ij + gamma |Q_ic|, below 1e-5) or KRR_BF16 /
- * KRR_FP16 (reduced-precision kernel values, float32 accumulation).
+ * KRR_FP16 (reduced-precision kernel values, float32 accumulation).  In 16
+ * bits, up to 8 dimensions and under the Gaussian kernel, the points are sorted
+ * in Morton instead of Hilbert order: which targets share a block decides the
+ * form their kernel values are rounded in.
  * The call may wait briefly for the point preparation (Hilbert sort and block
  * metadata) to read the block counts that size the product grids (single
  * columns in float32 of up to 16384 points up to 8 dimensions do not need
@@ -267,7 +271,10 @@ krr_status krr_points_create(krr_handle h, const float* X, int64_t N, int d,
  * Q, Y: DEVICE arrays, N x m column-major, 1 <= m <= 64; Y must not alias
  * Q.  Host arrays: KRR_ERR_INVALID_ARG.  The handle's product options
  * (KRR_OPT_TCGEN05, _DIRECT_TENSOR, _HIGHD_TCGEN05, _AUTOTUNE, the row
- * shards) apply as at the call.  No host synchronisation.  The products'
+ * shards) apply as at the call.  No host synchronisation, but for the first
+ * KRR_BF16 or KRR_FP16 product of a Gaussian point set of up to 8 dimensions,
+ * which sorts the points once more, in Morton order (see krr_kernel_mvp), and
+ * waits for the block counts (while capturing: KRR_ERR_INVALID_ARG).  The products'
  * scratch belongs to the point set: once a product of this (m, prec) has
  * run on it, a call allocates nothing and can be captured in a CUDA graph,
  * which stays valid until krr_points_destroy (the first call of a shape may

@@ -42,4 +42,9 @@ struct krr_points_s {
   krr_handle_s* h = nullptr;
   krr::Ctx ctx;
   krr::PointsDev P;
+  float sigma = 0.f;
+  // the same points in Morton order, for the products whose results depend on
+  // the order (order_decides); made by the first of them
+  krr::PointsDev morton;
+  bool has_morton = false;
 };

@@ -141,7 +141,7 @@ struct Ctx {
   // kernel values on the CUDA cores, the weighted sum on the tensor cores
   // (mvp_dirtc_kernel); false: the all-CUDA-core kernel mvp_dirm_kernel
   bool direct_tensor = true;
-  // sort points in Morton order (set while krr_mll_grad runs)
+  // sort points in Morton order (MortonScope)
   bool morton = false;
   // kernel function of every product and solve (KRR_KERNEL_*, krr_set_option)
   int kernel_family = 0;
@@ -264,12 +264,36 @@ constexpr double TUNE_MAX_BYTES = 1073741824.0;
 cudaError_t sub_context(Ctx& c, size_t k, Ctx** out);
 void release_context(Ctx& c);
 
+// Points prepared while one of these is on are sorted in Morton order.
+struct MortonScope {
+  Ctx& c;
+  const bool old;
+  MortonScope(Ctx& cc, bool on) : c(cc), old(cc.morton) { c.morton = old || on; }
+  ~MortonScope() { c.morton = old; }
+};
+// Whether the order of the points decides more than the order of a product's
+// sums.  In 16 bits it does where compact blocks take another form than the
+// others (the Gaussian, up to 8 dimensions): compact blocks hold the recentred
+// 2^E in f16 or bf16, the others 2^15 times the kernel value, and a target's
+// result differs between the two by the rounding of 16 bits.  Which targets
+// share a block is the sort's choice: with the points along the Hilbert curve
+// instead of the Morton curve the f16 products of 20,011 points in d = 4 and
+// 70,001 in d = 2 moved by 3.1e-4 (relative), bf16 by 2.5e-3, and those of
+// 16,385 normal points in d = 8 by up to 4e-5 through the two targets that are
+// alone in the last block.  Products in 16 bits therefore keep the Morton
+// order, and with it their results; float32 products differ by 4e-7 at most.
+inline bool order_decides(int kernel_family, int d, krr_precision prec) {
+  return prec != KRR_FP32 && kernel_family == KRR_KERNEL_GAUSSIAN && d <= 8;
+}
+
 // ---- prep.cu
 // Sort X (N x d row-major, device) along a Hilbert curve and pack the scaled,
 // tile-blocked structure-of-arrays copy.  `tag` names the workspace slots.
 // Under c.morton they are sorted in Morton order.
 cudaError_t prepare_points(Ctx& c, const float* X, int64_t N, int d, float sigma,
                            const char* tag, PointsDev& P, cudaStream_t st, bool read_counts = true);
+// X (N x d_in row-major, device) back from the packed copy, original order.
+cudaError_t unpack_points(const PointsDev& P, float* X, cudaStream_t st);
 // out[i] = in[perm[i]] (float columns, m of them, column stride N / Npad);
 // padded tail of each column set to zero.  qbad (may be null): per tile of SB
 // rows, 1 when a value is not below f16's largest in size (infinities and

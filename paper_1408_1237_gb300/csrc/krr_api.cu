@@ -508,6 +508,7 @@ krr_status krr_kernel_mvp(krr_handle h, const float* X, int64_t N, int d, float 
   // a shard leaves the other rows of Y as they were: a host Y goes up first
   if ((s = device_view(c, "stage.Y", Y, (size_t)N * m, sharded, st, &dY, &sY))) return s;
   PointsDev P;
+  MortonScope order(c, order_decides(c.kernel_family, d, prec));
   // a small single-column product needs no block counts on the host, hence no
   // wait for the preparation (4096 points: 70 us a call
   // with it and three product launches, 52 without)
@@ -571,6 +572,7 @@ krr_status krr_points_create(krr_handle h, const float* X, int64_t N, int d, flo
   krr_points_s* pts = new (std::nothrow) krr_points_s;
   if (!pts) return set_error(c, KRR_ERR_OOM, "%s: out of host memory", fn);
   pts->h = h;
+  pts->sigma = sigma;
   Ctx& pc = pts->ctx;
   pc.device = c.device;
   pc.num_sms = c.num_sms;
@@ -600,6 +602,28 @@ krr_status krr_points_create(krr_handle h, const float* X, int64_t N, int d, flo
   return KRR_OK;
 }
 
+// The points of a set in Morton order, from its packed copy (the caller's X may
+// be gone).  Waits once, for the block counts.
+static cudaError_t make_morton(Ctx& c, krr_points_s* pts, cudaStream_t st) {
+  Ctx& pc = pts->ctx;
+  void* X;
+  cudaError_t e = pc.ws.get("sort.x", sizeof(float) * (size_t)pts->P.N * pts->P.d_in, &X);
+  if (!e) e = unpack_points(pts->P, (float*)X, st);
+  if (e) return e;
+  const int family = pc.kernel_family;
+  pc.kernel_family = pts->P.kfam;  // the family at creation
+  pc.h_counts = c.h_counts;
+  {
+    MortonScope order(pc, true);
+    e = prepare_points(pc, (const float*)X, pts->P.N, pts->P.d_in, pts->sigma, "morton", pts->morton, st);
+  }
+  pc.h_counts = nullptr;
+  pc.kernel_family = family;
+  if (!e) pc.ws.release_prefix("sort.");
+  pts->has_morton = !e;
+  return e;
+}
+
 krr_status krr_kernel_mvp_points(krr_handle h, krr_points P, const float* Q, int m, float gamma, float* Y,
                                  krr_precision prec, void* stream) {
   NvtxRange nvtx_range("krr_kernel_mvp_points");
@@ -621,8 +645,17 @@ krr_status krr_kernel_mvp_points(krr_handle h, krr_points P, const float* Q, int
                      c.shard_count);
   Ctx& pc = P->ctx;
   copy_product_options(pc, c);
-  cudaError_t e = product_prepared(pc, P->P, Q, m, gamma, prec, Y, (cudaStream_t)stream);
-  if (e) return cuda_error(c, e, fn);
+  cudaStream_t st = (cudaStream_t)stream;
+  cudaError_t e;
+  const bool morton = order_decides(P->P.kfam, P->P.d_in, prec);
+  if (morton && !P->has_morton) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if ((e = cudaStreamIsCapturing(st, &cs))) return cuda_error(c, e, fn);
+    if (cs != cudaStreamCaptureStatusNone)
+      return set_error(c, KRR_ERR_INVALID_ARG, "%s: the first product in 16 bits cannot be captured", fn);
+    if ((e = make_morton(c, P, st))) return cuda_error(c, e, fn);
+  }
+  if ((e = product_prepared(pc, morton ? P->morton : P->P, Q, m, gamma, prec, Y, st))) return cuda_error(c, e, fn);
   return KRR_OK;
 }
 
@@ -666,6 +699,7 @@ krr_status krr_kernel_mvp_rect(krr_handle h, const float* Xt, int64_t Nt, const 
   } else {
     if (!Q) return set_error(c, KRR_ERR_INVALID_ARG, "%s: Q is NULL", fn);
     PointsDev T, S;
+    MortonScope order(c, order_decides(c.kernel_family, d, prec));
     if ((e = prepare_points(c, dXt, Nt, d, sigma, "pts_t", T, st))) return cuda_error(c, e, fn);
     if ((e = prepare_points(c, dXs, Ns, d, sigma, "pts_s", S, st))) return cuda_error(c, e, fn);
     void* qs;

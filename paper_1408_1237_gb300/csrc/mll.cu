@@ -343,11 +343,7 @@ extern "C" krr_status krr_mll_grad(krr_handle h, const float* X, int64_t N, int 
   // value at random (through the sums, and by 1e-6 through the last bits of
   // the solutions); the adjoint takes the direct form for every pair, so the
   // order costs it nothing
-  struct Order {
-    Ctx& c;
-    explicit Order(Ctx& cc) : c(cc) { c.morton = true; }
-    ~Order() { c.morton = false; }
-  } order(c);
+  MortonScope order(c, true);
   const int P = n_probes, nrhs = 1 + P, ncols = 2 * P + 1;
   float *dXin, *dy, *ddX = nullptr;
   bool sX, sy, sdX = false;

@@ -1,4 +1,4 @@
-// Point preparation (hot-path step A1): Hilbert-order sort, scaling and
+// Point preparation (hot-path step A1): Hilbert- or Morton-order sort, scaling and
 // tile-blocked packing of the points.
 //
 // The Gaussian of Eq. 2 becomes a base-2 exponential of scaled points:
@@ -496,6 +496,15 @@ __global__ void __launch_bounds__(TS)
   }
 }
 
+__global__ void unpack_kernel(const float* __restrict__ xs, int64_t N, int d_in, int d, const int* __restrict__ perm,
+                              float* __restrict__ X) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  const float* src = xs + i / TS * (int64_t)d * TS + i % TS;
+  float* row = X + (int64_t)perm[i] * d_in;
+  for (int k = 0; k < d_in; ++k) row[k] = src[(int64_t)k * TS];
+}
+
 // (Npad is a multiple of the block: no thread leaves early)
 __global__ void __launch_bounds__(TS)
     gather_kernel(const float* __restrict__ in, int64_t N, int m, const int* __restrict__ perm, int64_t Npad,
@@ -618,6 +627,12 @@ cudaError_t gather_sorted(const float* in, int64_t N, int m, const int* perm, in
                           float* out, cudaStream_t st, int* qbad) {
   if (Npad == 0) return cudaSuccess;
   gather_kernel<<<blocks_for(Npad, TS), TS, 0, st>>>(in, N, m, perm, Npad, out, qbad); count_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t unpack_points(const PointsDev& P, float* X, cudaStream_t st) {
+  if (P.N == 0) return cudaSuccess;
+  unpack_kernel<<<blocks_for(P.N, 256), 256, 0, st>>>(P.xs, P.N, P.d_in, P.d, P.perm, X); count_launch();
   return cudaGetLastError();
 }
 

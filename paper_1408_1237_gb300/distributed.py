@@ -3,7 +3,7 @@
 The product y = (K_hat + gamma I) q is the O(N^2) step that the paper runs
 on the GPU (Sec. 3.1); split over P ranks by target rows, each rank sums its
 rows against all sources (N^2 / P pairs) and one collective assembles y on
-every rank before the next Krylov step.  Rank k computes the Hilbert-ordered
+every rank before the next Krylov step.  Rank k computes the sorted
 super-blocks [k nsb / P, (k+1) nsb / P) of 256 targets (the library's
 KRR_OPT_SHARD_COUNT / KRR_OPT_SHARD_INDEX), writing its rows into a zeroed Y;
 the collective is a sum all-reduce of Y (rows a rank did not compute are
