@@ -170,7 +170,8 @@ struct Ctx {
   int prof_tensor_exp = 0;           // timed launches on the tensor-core exponent path
 };
 
-// Product shape key of the autotuner: kind ("mvp" or "acc"), sizes, columns,
+// Product shape key of the autotuner: kind ("mvp", "fine" for MvpOut::fine, or
+// "acc"), sizes, columns,
 // precision, kernel family and the planning context.
 std::string tune_key(const Ctx& c, const char* kind, const PointsDev& Tp, const PointsDev& Sp, int m,
                      int prec);
@@ -351,8 +352,9 @@ struct MvpOut {
   // not cancel (gather_sorted; null: none does, as in the solvers, whose
   // iteration stops on a product that is not finite wherever it appears)
   const int* qbad = nullptr;
-  // several columns take the tensor-core kernels' form that is as exact as the
-  // single-column kernels (the prediction product, in whose place it stands)
+  // several float32 columns take the tensor-core kernels' form that is as exact
+  // as the single-column kernels (the prediction product, in whose place it
+  // stands); the tcgen05 kernels have none and are left out
   bool fine = false;
   // y = alpha * (K_hat q + shift q) + beta * u, sorted order
   float alpha = 1.f, beta = 0.f;

@@ -808,11 +808,11 @@ Plan f32_plan(const Ctx& c, const PointsDev& Tp, const PointsDev& Sp) {
 // Source splits of the multi-column kernels (one CTA per super-block): the
 // tensor-core kernel over the expanded-form super-blocks, the CUDA-core
 // kernel over the direct-form ones, each planned for its own grid.
-Plan multi_plan_tc(const Ctx& c, const PointsDev& Tp, const PointsDev& Sp, krr_precision prec, int m) {
-  // two CTAs (of 128 targets) per super-block, at most two per SM (tensor memory)
+// fine (MvpOut::fine): the mma.sync kernel, whatever the handle's choice.
+Plan multi_plan_tc(const Ctx& c, const PointsDev& Tp, const PointsDev& Sp, krr_precision prec, int m, bool fine) {
   // one CTA per super-block (mma.sync kernel), or two of 128 targets with at
   // most two per SM (tcgen05 kernel: tensor memory)
-  return make_plan((tc5_on(c, prec, m, Tp) ? 2 : 1) * Tp.h_sb_nexp * NW, source_tiles(Sp), c.num_sms,
+  return make_plan((!fine && tc5_on(c, prec, m, Tp) ? 2 : 1) * Tp.h_sb_nexp * NW, source_tiles(Sp), c.num_sms,
                    c.plan_slots, c.split_scale, SETUP_MULTI);
 }
 // Multi-column products keep the tensor cores to d <= 8 (Gaussian); elsewhere
@@ -898,13 +898,13 @@ cudaError_t common_reserve(Ctx& c, const PointsDev& Tp, cudaStream_t st) {
 
 // Largest source-split count among the kernels of a product route at the
 // split scale in force (sizes the partial-sum buffers of a tuning candidate).
-int route_splits(const Ctx& c, const PointsDev& Tp, const PointsDev& Sp, int m, krr_precision prec) {
+int route_splits(const Ctx& c, const PointsDev& Tp, const PointsDev& Sp, int m, krr_precision prec, bool fine) {
   if (m == 1 && prec == KRR_FP32) {
     if (use_tcx(c, Tp)) return std::max(tcx_plan(c, Tp, Sp).splits, tcx_dir_plan(c, Tp, Sp).splits);
     if (Tp.d <= 8) return f32_plan(c, Tp, Sp).splits;
   }
   int s = multi_plan_dir(c, Tp, Sp).splits;
-  if (!multi_direct_only(Tp)) s = std::max(s, multi_plan_tc(c, Tp, Sp, prec, m).splits);
+  if (!multi_direct_only(Tp)) s = std::max(s, multi_plan_tc(c, Tp, Sp, prec, m, fine).splits);
   return s;
 }
 
@@ -916,7 +916,7 @@ int route_splits(const Ctx& c, const PointsDev& Tp, const PointsDev& Sp, int m, 
 // faster).  Split candidates whose partial sums would exceed TUNE_MAX_BYTES
 // are skipped.
 cudaError_t autotune_mvp(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, int m, krr_precision prec,
-                         cudaStream_t st, const std::string& key, bool tcgen05_only = false) {
+                         cudaStream_t st, const std::string& key, bool tcgen05_only = false, bool fine = false) {
   struct Restore {
     Ctx& c;
     bool prof;
@@ -940,6 +940,7 @@ cudaError_t autotune_mvp(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, int m
   }
   MvpOut o;
   o.out_f = (float*)yv;
+  o.fine = fine;
   const bool single = m == 1 && prec == KRR_FP32;
   auto run = [&]() {
     return single ? mvp_launch(c, Tp, Sp, (const float*)qv, nullptr, 0.f, prec, o, st)
@@ -964,12 +965,14 @@ cudaError_t autotune_mvp(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, int m
   // products up to 8 dimensions that would take the tensor-core exponent
   // path also try the packed CUDA-core kernel; multi-column Gaussian products
   // up to 8 dimensions try both kernels for compact blocks and both for
-  // direct-form blocks.  The handle's own variant is kept unless another is
-  // 2% faster.
+  // direct-form blocks (a fine product: the latter only).  The handle's own
+  // variant is kept unless another is 2% faster.
   const int cur = current_variant(c, prec, m, Tp);
   std::vector<int> variants{cur};
   if (tcgen05_only) {
     variants.push_back(cur ^ TV_TCGEN05);
+  } else if (fine) {
+    if (Tp.d <= 8 && Tp.kfam == KRR_KERNEL_GAUSSIAN) variants.push_back(cur ^ TV_DIRECT_TENSOR);
   } else if (single && Tp.d <= 8 && use_tcx(c, Tp)) {
     variants.push_back(cur & ~TV_TENSOR_EXP);
   } else if (!single && Tp.d <= 8 && Tp.kfam == KRR_KERNEL_GAUSSIAN) {
@@ -1003,7 +1006,7 @@ cudaError_t autotune_mvp(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, int m
     {
       TuneScope ts(c, s);
       VariantScope vs(c, key);
-      if (s > 1.0 && 8.0 * route_splits(c, Tp, Sp, m, prec) * m * (double)Tp.Npad > TUNE_MAX_BYTES)
+      if (s > 1.0 && 8.0 * route_splits(c, Tp, Sp, m, prec, fine) * m * (double)Tp.Npad > TUNE_MAX_BYTES)
         continue;
     }
     float ms;
@@ -1350,17 +1353,16 @@ cudaError_t mvp_multi_reserve(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, 
   const bool direct_only = multi_direct_only(Tp);
   cudaError_t e = direct_only ? common_reserve(c, Tp, st) : mvp_reserve(c, Tp, Sp, st);
   if (e) return e;
-  const Plan pt = multi_plan_tc(c, Tp, Sp, prec, m), pd = multi_plan_dir(c, Tp, Sp);
+  const Plan pt = multi_plan_tc(c, Tp, Sp, prec, m, false), pd = multi_plan_dir(c, Tp, Sp);
   void* v;
   if ((e = c.ws.get("mvp.partm", sizeof(double) * pt.splits * (size_t)m * Tp.Npad, &v))) return e;
   if ((e = c.ws.get("mvp.partd", sizeof(double) * pd.splits * (size_t)m * Tp.Npad, &v))) return e;
   MvpParams p{};
   p.nblk = Tp.nsb;
   if (use_dirtc(c, Tp)) {
-    for (bool fine : {false, true})
-      if ((e = mvp_dirtc_partials(c, Tp, Sp, nullptr, m, prec, pd.splits, pd.tiles_per_split, multi_nexp(Tp),
-                                  nullptr, nullptr, nullptr, nullptr, fine, st, true)))
-        return e;
+    if ((e = mvp_dirtc_partials(c, Tp, Sp, nullptr, m, prec, pd.splits, pd.tiles_per_split, multi_nexp(Tp),
+                                nullptr, nullptr, nullptr, nullptr, false, st, true)))
+      return e;
   } else if ((e = dirm_dispatch(p, Tp.d, Tp.kfam, nullptr, 0, m, SB / 32, multi_nexp(Tp), pd, st, false))) {
     return e;
   }
@@ -1368,11 +1370,8 @@ cudaError_t mvp_multi_reserve(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, 
   if (tc5_on(c, prec, m, Tp))
     return mvp_umma_partials(c, Tp, Sp, nullptr, m, prec == KRR_FP32, prec == KRR_BF16, pt.splits,
                              pt.tiles_per_split, nullptr, nullptr, nullptr, nullptr, st, true);
-  for (bool fine : {false, true})
-    if ((e = mvp_tc_partials(c, Tp, Sp, nullptr, m, prec, fine, pt.splits, pt.tiles_per_split, nullptr, nullptr,
-                             nullptr, nullptr, st, true)))
-      return e;
-  return cudaSuccess;
+  return mvp_tc_partials(c, Tp, Sp, nullptr, m, prec, false, pt.splits, pt.tiles_per_split, nullptr, nullptr,
+                         nullptr, nullptr, st, true);
 }
 
 // One column against a pass of 2 to 8, 16 columns on GB300: 131,072 points,
@@ -1393,9 +1392,10 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, c
                              cudaStream_t st) {
   if (Tp.N == 0) return cudaSuccess;
   if (Tp.d < 1 || (Tp.d > 8 && Tp.d % 16) || Tp.d > 64 || m < 1 || m > MAX_COLS) return cudaErrorNotSupported;
-  const std::string key = tune_key(c, "mvp", Tp, Sp, m, prec);
+  const bool fine = o.fine && prec == KRR_FP32;
+  const std::string key = tune_key(c, fine ? "fine" : "mvp", Tp, Sp, m, prec);
   if (can_tune(c, st) && !c.tune_cache.count(key)) {
-    cudaError_t te = autotune_mvp(c, Tp, Sp, m, prec, st, key);
+    cudaError_t te = autotune_mvp(c, Tp, Sp, m, prec, st, key, false, fine);
     if (te) return te;
   }
   TuneScope scope(c, tuned_scale(c, key));
@@ -1417,7 +1417,7 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, c
   p.s = Sp.scale;
   p.active = o.active;
   p.part_stride = (int64_t)m * Tp.Npad;
-  const Plan pt = multi_plan_tc(c, Tp, Sp, prec, m), pd = multi_plan_dir(c, Tp, Sp);
+  const Plan pt = multi_plan_tc(c, Tp, Sp, prec, m, fine), pd = multi_plan_dir(c, Tp, Sp);
   const bool direct_only = multi_direct_only(Tp);
   const int64_t nexp = multi_nexp(Tp);
   cudaError_t e = direct_only ? common_reserve(c, Tp, st) : mvp_reserve(c, Tp, Sp, st);
@@ -1460,12 +1460,13 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, c
   }
   // expanded-form super-blocks: all columns on the tensor cores (float32
   // products of more than 8 columns: P Q by tcgen05 in mvp_umx_kernel; the
-  // others: mma.sync; KRR_OPT_TCGEN05 overrides)
+  // others: mma.sync; KRR_OPT_TCGEN05 overrides).  A fine product has its form
+  // in the mma.sync kernel only.
   if (nexp > 0) {
-    e = tc5_on(c, prec, m, Tp)
+    e = !fine && tc5_on(c, prec, m, Tp)
             ? mvp_umma_partials(c, Tp, Sp, Q, m, prec == KRR_FP32, prec == KRR_BF16, pt.splits,
                                 pt.tiles_per_split, (double*)part, p.fac, o.active, o.qbad, st)
-            : mvp_tc_partials(c, Tp, Sp, Q, m, prec, o.fine, pt.splits, pt.tiles_per_split, (double*)part,
+            : mvp_tc_partials(c, Tp, Sp, Q, m, prec, fine, pt.splits, pt.tiles_per_split, (double*)part,
                               p.fac, o.active, o.qbad, st);
     if (e) return e;
   }
@@ -1481,7 +1482,7 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, c
     }
     if (use_dirtc(c, Tp)) {
       if ((e = mvp_dirtc_partials(c, Tp, Sp, Q, m, prec, pd.splits, pd.tiles_per_split, nexp, p.tn_exp,
-                                  (double*)partd, p.fac, o.active, o.fine, dst, false)))
+                                  (double*)partd, p.fac, o.active, fine, dst, false)))
         return e;
     } else if ((e = dirm_dispatch(p, Tp.d, Tp.kfam, Q, Sp.Npad, m, SB / 32, nexp, pd, dst, true))) {
       return e;
