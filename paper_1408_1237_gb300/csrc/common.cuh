@@ -147,6 +147,25 @@ __device__ __forceinline__ double f2d(float v) {
   return (double)v;
 }
 
+constexpr uint32_t TF32_MASK = 0xFFFFE000u;  // clears the 13 mantissa bits tf32 drops
+constexpr uint32_t TF32_HALF = 0x1000u;      // half a unit of tf32's last place
+
+// v rounded to tf32, half away from zero.  (The largest finite weights keep
+// their value: rounding up would carry into infinity.)
+__device__ __forceinline__ uint32_t tf32_hi(float v) {
+  const uint32_t u = __float_as_uint(v), up = u + TF32_HALF;
+  return ((up & 0x7F800000u) == 0x7F800000u ? u : up) & TF32_MASK;
+}
+
+// d += a b, tf32 operands.
+__device__ __forceinline__ void mma_1688_tf32(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 fadd2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 fmul2(float2 a, float2 b) { return __fmul2_rn(a, b); }

@@ -1374,10 +1374,14 @@ cudaError_t mvp_multi_reserve(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, 
                          nullptr, nullptr, st, true);
 }
 
-// One column against a pass of 2 to 8, 16 columns on GB300: 131,072 points,
-// d = 3, 2.51 ms against 4.9 to 5.3, 5.8; 20,000 points 148 us against 310 to
-// 322, 440; d = 8, 16,384 points 158 against 339 to 352, 479.  So two columns
-// tie and three gain 1.4 times in one pass.  Above 8 dimensions the pass takes
+// One column against a pass of 2, 3, 8, 16 columns on GB300: d = 3, 131,072
+// points 2.14 ms against 5.08, 5.10, 5.29, 8.97, 65,541 targets of 20,011
+// sources 295 us against 617, 619, 642, 945, 20,000 points 147 us against 265,
+// 264, 269, 348 (sigma = 0.3: 148 against 186, 186, 200, 315); d = 4, 150,000
+// of 20,000 527 us against 1161, 1164, 1248, 2077; d = 5, 60,000 points 0.94 ms
+// against 1.82, 1.83, 2.13, 2.92; d = 8, 16,384 points 133 us against 266, 267,
+// 269, 323.  So two columns tie and three gain 1.3 times or more in one pass.
+// Above 8 dimensions the pass takes
 // the direct form, where a single column has the tensor cores on compact
 // blocks: d = 16, 16,384 points 134 us against 422 up to 4 columns, 488 up to
 // 8, 749 at 16.

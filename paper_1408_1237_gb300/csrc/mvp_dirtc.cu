@@ -59,8 +59,6 @@ constexpr int DT_THREADS = 512;            // 16 warps: one m-tile of 16 targets
 constexpr int DT_RS = 2;                   // raw stages
 constexpr int QS = 264;                    // halves per f16 weight row of a work buffer (256 + pad)
 constexpr int QSW = 260;                   // words per tf32 weight row (256 + pad: conflict-free)
-constexpr uint32_t TF32_MASK = 0xFFFFE000u;  // clears the 13 mantissa bits tf32 drops
-constexpr uint32_t TF32_HALF = 0x1000u;      // half a unit of tf32's last place
 constexpr int FOLD = 64;                     // sources per accumulation of Ph Qh
 constexpr float F16_OFFSET = 15.f;         // f16 kernel values are 2^15 P
 constexpr float kLog2eDt = 1.4426950408889634f;
@@ -125,21 +123,6 @@ __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4],
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
   }
-}
-
-__device__ __forceinline__ void mma_1688_tf32(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-      "{%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// v rounded to tf32, half away from zero.  (The largest finite weights keep
-// their value: rounding up would carry into infinity.)
-__device__ __forceinline__ uint32_t tf32_hi(float v) {
-  const uint32_t u = __float_as_uint(v), up = u + TF32_HALF;
-  return ((up & 0x7F800000u) == 0x7F800000u ? u : up) & TF32_MASK;
 }
 
 // Kernel values of two pairs from their squared raw distances, times 2^off.

@@ -238,12 +238,37 @@ __device__ __forceinline__ float kv_value(const float (&h)[D + 1], const float (
   return v;
 }
 
-// SPLIT: 0 single operands; 1 hi + lo; 2 hi + lo with Ph Qh in fresh
-// accumulators every FOLD sources (the tensor cores truncate when they
-// accumulate) and the small products in accumulators of their own, where it
-// takes the place of single-column products.  Relative error at 131,072 points
-// in the cube 1.5e-6 with 1 and 2.8e-7 with 2 (2.5e-7 for the single-column
-// kernels), for 5 to 9% more time.
+// SPLIT: how P Q is held.
+//  0: single f16 or bf16 operands;
+//  1: f16 hi + lo.  Weights from 65,520 on are infinite in f16, and kernel
+//     values below 2^-25 are zero;
+//  2: tf32 hi + lo, where it takes the place of single-column products: their
+//     range of weights and kernel values, which a prediction needs (weights of
+//     any size, targets away from all sources, no diagonal term).  Ph Qh goes
+//     into fresh accumulators every FOLD sources (the tensor cores truncate when
+//     they accumulate) and the two small products into accumulators of their
+//     own.  A tf32 A operand wants the columns t and t + 4 where the exponent's
+//     accumulator has 2t and 2t + 1, so sources 2t and 2t + 1 take those places
+//     in P and Q alike.  The weights stay in the raw stage, in rows of 264 words
+//     (64-bit reads without bank conflicts), and are split when read, which the
+//     m-tiles of a warp share; a stage is refilled one step later for that, so
+//     there is one more.
+// Relative error of products of N(0, 1) weights at 131,072 points in the cube:
+// 1.5e-6 with 1; 65,541 targets and 20,011 sources: 3.0e-7 with 2, 2.2e-7 for
+// single columns.  A tf32 MMA contracts half as many sources in the same time,
+// and far fewer kernel values are zeros of tf32 than of f16, so 2 takes 619 us
+// for 4 columns there (f16 operands: 497, four single columns: 1180).
+template <int SPLIT>
+constexpr int tc_stages() { return SPLIT == 2 ? RS + 1 : RS; }
+template <int SPLIT>
+constexpr int tc_qrow() { return SPLIT == 2 ? TS + 8 : TS; }  // words from one weight row of a stage to the next
+template <int D, int SPLIT>
+constexpr size_t tc_smem_bytes(int m, int mc) {
+  return sizeof(float) * tc_stages<SPLIT>() * (D * TS + m * tc_qrow<SPLIT>()) +
+         sizeof(uint32_t) * 2 * TS * ExpLayout<D>::KV_STRIDE_W +
+         (SPLIT == 2 ? 0 : sizeof(uint32_t) * 2 * (SPLIT ? 2 : 1) * mc * 132);
+}
+
 template <int D, int MT, int NRT, int SPLIT, bool BF>
 __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
   using L = ExpLayout<D>;
@@ -251,11 +276,12 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
   constexpr int W = D + 1;
   constexpr int MC = 8 * NRT;  // padded right-hand sides
   constexpr int QSTRIDE_W = 132;  // words per column of a source tile (256 halves + pad)
+  constexpr int STAGES = tc_stages<SPLIT>(), QROW = tc_qrow<SPLIT>();
   extern __shared__ __align__(128) float smem[];
   const int nthreads = blockDim.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
-  __shared__ __align__(8) uint64_t bars[RS];
+  __shared__ __align__(8) uint64_t bars[STAGES];
   __shared__ volatile int abort_flag;
   __shared__ uint32_t live[LIVE_WORDS];
   __shared__ int live_n;
@@ -263,10 +289,10 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
   const int64_t nexp = *p.tn_exp;
   if ((int64_t)blockIdx.x >= nexp) return;  // direct-form blocks: CUDA-core kernel
 
-  const int raw_floats = (D + p.m) * TS;
-  float* raw = smem;                                                  // RS stages
-  uint32_t* kvb = reinterpret_cast<uint32_t*>(smem + RS * raw_floats);  // 2 x TS x KV_STRIDE_W
-  uint32_t* qb = kvb + 2 * TS * L::KV_STRIDE_W;                         // 2 x (SPLIT?2:1) x MC x QSTRIDE_W
+  const int raw_floats = D * TS + p.m * QROW;
+  float* raw = smem;                                                        // STAGES stages
+  uint32_t* kvb = reinterpret_cast<uint32_t*>(smem + STAGES * raw_floats);  // 2 x TS x KV_STRIDE_W
+  uint32_t* qb = kvb + 2 * TS * L::KV_STRIDE_W;                             // 2 x (SPLIT?2:1) x MC x QSTRIDE_W (not SPLIT 2)
   constexpr int QBUF_W = (SPLIT ? 2 : 1) * MC * QSTRIDE_W;
 
   const int64_t blk = p.torder[blockIdx.x];
@@ -314,7 +340,7 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
 
   // acc: P Q of the tile (SPLIT 2: Ph Qh of the current FOLD sources);
   // low: SPLIT 2, Pl Qh + Ph Ql of the tile
-  constexpr int FOLD = 64;
+  constexpr int FOLD = 64;  // (SPLIT 2)
   float acc[MT][NRT][4], low[MT][NRT][4];
   float S[MT][NRT][4], C[MT][NRT][4];
 #pragma unroll
@@ -325,20 +351,20 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
       for (int e = 0; e < 4; ++e) acc[mt][rt][e] = low[mt][rt][e] = S[mt][rt][e] = C[mt][rt][e] = 0.f;
 
   auto issue = [&](int r) {
-    const int stage = r % RS;
+    const int stage = r % STAGES;
     const int64_t tile = t_begin + tiles.pop();
     float* dst = raw + stage * raw_floats;
-    mbar_arrive_expect_tx(&bars[stage], (uint32_t)raw_floats * 4);
+    mbar_arrive_expect_tx(&bars[stage], (uint32_t)((D + p.m) * TS) * 4);
     bulk_g2s(dst, p.xs + tile * (int64_t)D * TS, D * TS * 4, &bars[stage]);
     for (int c = 0; c < p.m; ++c)
-      bulk_g2s(dst + (D + c) * TS, p.Q + (int64_t)c * p.Ns_pad + tile * (int64_t)TS, TS * 4,
+      bulk_g2s(dst + D * TS + c * QROW, p.Q + (int64_t)c * p.Ns_pad + tile * (int64_t)TS, TS * 4,
                &bars[stage]);
   };
 
   // CTA-wide transform of raw tile r into buffer b: source K-vectors and the
   // weights in half precision (hi, and lo when split)
   auto transform = [&](int r, int b) {
-    const float* rs = raw + (r % RS) * raw_floats;
+    const float* rs = raw + (r % STAGES) * raw_floats;
     uint32_t* kv = kvb + b * TS * L::KV_STRIDE_W;
     uint32_t* qq = qb + b * QBUF_W;
     for (int j = tid; j < TS; j += nthreads) {
@@ -369,6 +395,7 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
       for (int w = 0; w < L::KV / 2; ++w)
         kv[j * L::KV_STRIDE_W + w] = (uint32_t)hv[2 * w] | ((uint32_t)hv[2 * w + 1] << 16);
     }
+    if (SPLIT == 2) return;
     // weights: column c of the tile as halves at qq[c*QSTRIDE_W*2 + j]
     uint16_t* qh = reinterpret_cast<uint16_t*>(qq);
     uint16_t* ql = qh + MC * QSTRIDE_W * 2;
@@ -386,13 +413,13 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
 
   if (tid == 0) {
     abort_flag = 0;
-    for (int st = 0; st < RS; ++st) mbar_init(&bars[st], 1);
+    for (int st = 0; st < STAGES; ++st) mbar_init(&bars[st], 1);
     fence_barrier_init();
   }
   __syncthreads();
   int issued = 0;
   if (tid == 0)
-    for (; issued < min(RS, nt); ++issued) issue(issued);
+    for (; issued < min(STAGES, nt); ++issued) issue(issued);
   if (nt > 0) {
     const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bars[0], 0));
     if (!ok) {
@@ -405,14 +432,15 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
   }
 
   for (int r = 0; r < nt && !abort_flag; ++r) {
-    // raw stage r % RS was consumed by transform(r); refill it with tile r + RS
-    if (tid == 0 && r + RS < nt) {
+    // raw stage r % RS was consumed by transform(r) (SPLIT 2: stage
+    // (r - 1) % STAGES by step r - 1): refill it with tile r + RS
+    if (tid == 0 && issued == r + RS && issued < nt) {
       fence_proxy_async_smem();
-      issue(r + RS);
+      issue(issued);
       ++issued;
     }
     if (r + 1 < nt) {
-      const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bars[(r + 1) % RS], ((r + 1) / RS) & 1));
+      const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bars[(r + 1) % STAGES], ((r + 1) / STAGES) & 1));
       if (!ok) {
         abort_flag = 1;
         if (lane == 0) atomicExch(p.err, DEV_TIMEOUT);
@@ -436,16 +464,30 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
           bfr[nt2][ks][1] = kv[j * L::KV_STRIDE_W + 8 * ks + t + 4];
         }
       }
-      // weights operand for each group of 8 right-hand sides
-      uint32_t qfh[NRT][2], qfl[NRT][2];
+      // weights operand for each group of 8 right-hand sides (SPLIT 2: of each
+      // half, sources 2t and 2t + 1)
+      uint32_t qfh[NRT][SPLIT == 2 ? 4 : 2], qfl[NRT][SPLIT == 2 ? 4 : 2];
 #pragma unroll
       for (int rt = 0; rt < NRT; ++rt) {
         const int c = rt * 8 + g;
-        qfh[rt][0] = qh[c * QSTRIDE_W + kk * 8 + t];
-        qfh[rt][1] = qh[c * QSTRIDE_W + kk * 8 + t + 4];
-        if (SPLIT) {
-          qfl[rt][0] = ql[c * QSTRIDE_W + kk * 8 + t];
-          qfl[rt][1] = ql[c * QSTRIDE_W + kk * 8 + t + 4];
+        if constexpr (SPLIT == 2) {
+          const float* qr = raw + (r % STAGES) * raw_floats + D * TS + c * QROW + kk * 16 + 2 * t;
+          const float2 zero = make_float2(0.f, 0.f);
+          const float2 q0 = c < p.m ? *reinterpret_cast<const float2*>(qr) : zero;
+          const float2 q1 = c < p.m ? *reinterpret_cast<const float2*>(qr + 8) : zero;
+          const float v[4] = {q0.x, q0.y, q1.x, q1.y};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            qfh[rt][e] = tf32_hi(v[e]);
+            qfl[rt][e] = __float_as_uint(v[e] - __uint_as_float(qfh[rt][e]));
+          }
+        } else {
+          qfh[rt][0] = qh[c * QSTRIDE_W + kk * 8 + t];
+          qfh[rt][1] = qh[c * QSTRIDE_W + kk * 8 + t + 4];
+          if (SPLIT) {
+            qfl[rt][0] = ql[c * QSTRIDE_W + kk * 8 + t];
+            qfl[rt][1] = ql[c * QSTRIDE_W + kk * 8 + t + 4];
+          }
         }
       }
 #pragma unroll
@@ -464,25 +506,46 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
           pv[e] = ex2(e0[e]);
           pv[4 + e] = ex2(e1[e]);
         }
-        uint32_t ph[4];
-        ph[0] = H::pack(pv[0], pv[1]);
-        ph[1] = H::pack(pv[2], pv[3]);
-        ph[2] = H::pack(pv[4], pv[5]);
-        ph[3] = H::pack(pv[6], pv[7]);
-        uint32_t pl[4];
-        if (SPLIT) {
+        if constexpr (SPLIT == 2) {
 #pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            const float2 hv = H::unpack(ph[w]);
-            pl[w] = H::pack(pv[2 * w] - hv.x, pv[2 * w + 1] - hv.y);
+          for (int hf = 0; hf < 2; ++hf) {
+            // rows g, g + 8 of source 2t, then of 2t + 1 (P <= 2^EXPANDED_R2:
+            // rounding up does not overflow)
+            const float v[4] = {pv[4 * hf], pv[4 * hf + 2], pv[4 * hf + 1], pv[4 * hf + 3]};
+            uint32_t ah[4], al[4];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+              ah[w] = (__float_as_uint(v[w]) + TF32_HALF) & TF32_MASK;
+              al[w] = __float_as_uint(v[w] - __uint_as_float(ah[w]));
+            }
+#pragma unroll
+            for (int rt = 0; rt < NRT; ++rt) {
+              mma_1688_tf32(acc[mt][rt], ah, qfh[rt][2 * hf], qfh[rt][2 * hf + 1]);
+              mma_1688_tf32(low[mt][rt], al, qfh[rt][2 * hf], qfh[rt][2 * hf + 1]);
+              mma_1688_tf32(low[mt][rt], ah, qfl[rt][2 * hf], qfl[rt][2 * hf + 1]);
+            }
           }
-        }
-#pragma unroll
-        for (int rt = 0; rt < NRT; ++rt) {
-          mma16816<BF>(acc[mt][rt], ph, qfh[rt][0], qfh[rt][1]);
+        } else {
+          uint32_t ph[4];
+          ph[0] = H::pack(pv[0], pv[1]);
+          ph[1] = H::pack(pv[2], pv[3]);
+          ph[2] = H::pack(pv[4], pv[5]);
+          ph[3] = H::pack(pv[6], pv[7]);
+          uint32_t pl[4];
           if (SPLIT) {
-            mma16816<BF>(SPLIT == 2 ? low[mt][rt] : acc[mt][rt], pl, qfh[rt][0], qfh[rt][1]);
-            mma16816<BF>(SPLIT == 2 ? low[mt][rt] : acc[mt][rt], ph, qfl[rt][0], qfl[rt][1]);
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+              const float2 hv = H::unpack(ph[w]);
+              pl[w] = H::pack(pv[2 * w] - hv.x, pv[2 * w + 1] - hv.y);
+            }
+          }
+#pragma unroll
+          for (int rt = 0; rt < NRT; ++rt) {
+            mma16816<BF>(acc[mt][rt], ph, qfh[rt][0], qfh[rt][1]);
+            if (SPLIT) {
+              mma16816<BF>(acc[mt][rt], pl, qfh[rt][0], qfh[rt][1]);
+              mma16816<BF>(acc[mt][rt], ph, qfl[rt][0], qfl[rt][1]);
+            }
           }
         }
       }
@@ -512,7 +575,7 @@ __global__ void __launch_bounds__(256) mvp_tc_kernel(const TcParams p) {
   }
   if (abort_flag) {
     if (tid == 0)
-      for (int r = 0; r < issued; ++r) mbar_wait_bounded(&bars[r % RS], (r / RS) & 1);
+      for (int r = 0; r < issued; ++r) mbar_wait_bounded(&bars[r % STAGES], (r / STAGES) & 1);
     __syncthreads();
     return;
   }
@@ -2302,17 +2365,14 @@ cudaError_t tch_launch_typed(const TcParams& p, int splits, cudaStream_t st, boo
 
 template <int D, int MT, int NRT, int SPLIT, bool BF>
 cudaError_t launch(const TcParams& p, int splits, int warps, cudaStream_t st, bool dry) {
-  using L = ExpLayout<D>;
   constexpr int MC = 8 * NRT;
-  const size_t shm = sizeof(float) * RS * (D + p.m) * TS + sizeof(uint32_t) * 2 * TS * L::KV_STRIDE_W +
-                     sizeof(uint32_t) * 2 * (SPLIT ? 2 : 1) * MC * 132;
+  const size_t shm = tc_smem_bytes<D, SPLIT>(p.m, MC);
   static bool done[128] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 128 && !done[dev]) {
     // sized for the largest m of this instance
-    const size_t shm_max = sizeof(float) * RS * (D + MC) * TS + sizeof(uint32_t) * 2 * TS * L::KV_STRIDE_W +
-                           sizeof(uint32_t) * 2 * (SPLIT ? 2 : 1) * MC * 132;
+    const size_t shm_max = tc_smem_bytes<D, SPLIT>(MC, MC);
     cudaError_t e = cudaFuncSetAttribute(mvp_tc_kernel<D, MT, NRT, SPLIT, BF>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_max);
     if (e) return e;
@@ -2372,7 +2432,7 @@ cudaError_t mvp_tc_partials(Ctx& c, const PointsDev& T, const PointsDev& S, cons
   p.tbox_t = T.tbox;
   p.tbox_s = S.tbox;
   p.qbad = qbad;
-  p.cut = prec == KRR_BF16 ? CUT_F32 : CUT_F16;  // P as f16 (hi + lo)
+  p.cut = prec == KRR_BF16 || fine ? CUT_F32 : CUT_F16;  // P as f16 (hi + lo), but for bf16 and tf32
   switch (T.d) {
     case 1: return dispatch_prec<1>(p, splits, prec, fine, st, dry);
     case 2: return dispatch_prec<2>(p, splits, prec, fine, st, dry);

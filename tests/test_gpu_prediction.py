@@ -54,3 +54,59 @@ def test_kernel_options_do_not_change_a_prediction(K, oracle_mod, m):
         assert torch.equal(K.krr_kernel_mvp_rect(*dev, 0.3, handle=h), tuned)
     for y in (ys[0], tuned):
         assert errors(oracle_mod, Xt, Xs, Q[:2], y[:2].cpu().numpy(), 0.3).max() <= 1e-5
+
+
+# The bar of the float32 products is 1e-5.  A pass of several columns drops
+# Pl Ql and sums three tf32 products per term: 3 * 2^-20 on top of the error of
+# the same columns alone.  Ten widths out the exponent is 72 and more: rounding
+# its f16 hi + lo operands (72 * 2^-23, and 2^-23 * 17 * 2.8 for the cross term)
+# and truncating in its float32 accumulator (120 * 2^-23) moves it by at most
+# 4e-5, single columns too.
+TOL, SPLIT, TOL_FAR = 1e-5, 3 * 2.0 ** -20, 4e-5
+
+
+@pytest.mark.parametrize("m", [1, 3, 4, 8, 9, 16, 17])
+@pytest.mark.parametrize("scale", [1e-6, 1.0, 1e5, 1e30, "mixed"])
+def test_weights_of_any_size(K, oracle_mod, m, scale):
+    """Compact blocks (sigma 0.3), direct-form blocks (0.02) and both (0.14)."""
+    import torch
+    Xt, Xs, rng = _clouds(3, 1801, 1501, m)
+    Q = rng.standard_normal((m, 1501)).astype(np.float32)
+    Q *= np.float32(scale) if scale != "mixed" else np.float32(10.0) ** rng.uniform(-6, 5, Q.shape).astype(np.float32)
+    Qd = torch.from_numpy(Q if m > 1 else Q[0]).cuda()
+    for sigma in (0.3, 0.14, 0.02):
+        y = K.krr_kernel_mvp_rect(torch.from_numpy(Xt).cuda(), torch.from_numpy(Xs).cuda(), Qd, sigma)
+        y = y.cpu().numpy().reshape(m, -1)
+        for c in {0, m // 2, m - 1}:
+            assert errors(oracle_mod, Xt, Xs, Q[c], y[c], sigma)[0] <= TOL, (sigma, c)
+
+
+@pytest.mark.parametrize("d,sigma", [(1, 0.05), (2, 0.15), (3, 0.2), (4, 0.25), (8, 0.5)])
+@pytest.mark.parametrize("m", [3, 16])
+def test_targets_away_from_all_sources(K, oracle_mod, m, d, sigma):
+    import torch
+    Xt0, Xs, rng = _clouds(d, 301, 1501, d)
+    Q = rng.standard_normal((m, 1501)).astype(np.float32)
+    Xsd, Qd = torch.from_numpy(Xs).cuda(), torch.from_numpy(Q).cuda()
+    for out in (0, 2, 3, 4, 5, 6, 10):
+        Xt = (1.5 * sigma * Xt0).astype(np.float32)  # one compact block and a remainder
+        Xt[:, 0] += np.float32(1.0 + out * sigma)
+        Xtd = torch.from_numpy(Xt).cuda()
+        got = errors(oracle_mod, Xt, Xs, Q[:3], K.krr_kernel_mvp_rect(Xtd, Xsd, Qd, sigma)[:3].cpu().numpy(), sigma)
+        alone = np.stack([K.krr_kernel_mvp_rect(Xtd, Xsd, Qd[c].contiguous(), sigma).cpu().numpy() for c in range(3)])
+        one = errors(oracle_mod, Xt, Xs, Q[:3], alone, sigma)
+        assert got.max() <= (TOL if out <= 6 else TOL_FAR), (out, got, one)
+        if out <= 3:
+            assert (got <= one + SPLIT).all(), (out, got, one)
+
+
+def test_infinite_weight_stays_in_its_column(K):
+    import torch
+    Xt, Xs, rng = _clouds(2, 700, 1100, 5)
+    dev = [torch.from_numpy(a).cuda() for a in (Xt, Xs)]
+    Q = torch.from_numpy(rng.standard_normal((3, 1100)).astype(np.float32)).cuda()
+    y = K.krr_kernel_mvp_rect(*dev, Q, 0.2)
+    Q[0, 17] = float("inf")
+    z = K.krr_kernel_mvp_rect(*dev, Q, 0.2)
+    torch.cuda.synchronize()
+    assert torch.equal(y[1:], z[1:]) and not torch.isfinite(z[0]).any()
