@@ -100,7 +100,7 @@ struct Ctx {
   Workspace ws;
   int* d_err = nullptr;        // device error word (DevErr)
   int* h_status = nullptr;     // pinned host mirror for status reads
-  int* h_counts = nullptr;     // two pinned words the preparation's block counts land in (null: copied)
+  int* h_counts = nullptr;     // two pinned words the block counts of a waiting preparation land in (null: copied)
   std::string last_error;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   // solver work runs on this non-blocking stream (capturable), joined to the

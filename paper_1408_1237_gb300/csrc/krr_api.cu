@@ -130,7 +130,7 @@ cudaError_t sub_context(Ctx& c, size_t k, Ctx** out) {
     s->aux = c.aux;
     s->ev_fork = c.ev_fork;
     s->ev_join = c.ev_join;
-    s->h_counts = c.h_counts;  // a preparation waits for its counts, so the words can be shared
+    s->h_counts = c.h_counts;  // whoever writes the words waits for them
     cudaError_t e = cudaMalloc(&s->d_err, sizeof(int));
     if (!e) e = cudaMemset(s->d_err, 0, sizeof(int));
     if (e) {

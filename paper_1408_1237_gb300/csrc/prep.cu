@@ -746,9 +746,11 @@ cudaError_t prepare_points(Ctx& c, const float* X, int64_t N, int d, float sigma
                                                allow_expanded_sb, po); count_launch();
   // the block counts size the product grids: the host reads them once (a short
   // wait for the preparation; never inside a graph capture), from pinned words
-  // that the kernel writes, or by copies where the context has none
+  // that the kernel writes, or by copies where the context has none.  Without
+  // the wait the words are left alone: the kernel may run while another
+  // preparation on the handle waits for its own counts.
   int counts[2] = {0, 0};
-  int* hc = c.h_counts;
+  int* hc = read_counts ? c.h_counts : nullptr;
   order_kernel<<<2, SCAN_THREADS, 0, st>>>(OrderArgs{(const int*)flag, P.nblk, P.order, P.n_exp, hc},
                                            OrderArgs{P.sb_flag, P.nsb, P.sb_order, P.sb_nexp, hc ? hc + 1 : nullptr});
   count_launch();

@@ -119,3 +119,27 @@ def test_points_argument_checks(K):
     finally:
         h1.close()
         h2.close()
+
+
+def test_point_sets_created_beside_products_on_another_stream(K):
+    """A point set reads its own block counts while the handle's small products
+    (which wait for nothing) run on another stream with other counts: a cloud
+    of wide blocks beside one of compact blocks, and the other way round."""
+    import torch
+    rng = np.random.default_rng(21)
+    compact, wide = _dev(0.01 * rng.random((4096, 3)).astype(np.float32)), _dev(rng.random((20000, 3)).astype(np.float32))
+    q, Q = _dev(rng.standard_normal(4096).astype(np.float32)), _dev(rng.standard_normal((2, 20000)).astype(np.float32))
+    sigma = 0.02
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    with K.Handle() as h:
+        want_q = K.krr_kernel_mvp(compact, q, sigma, 1e-3, handle=h)
+        want_Q = K.krr_kernel_mvp(wide, Q, sigma, 1e-3, handle=h)
+        torch.cuda.synchronize()
+        for _ in range(60):
+            ys = [K.krr_kernel_mvp(compact, q, sigma, 1e-3, handle=h, stream=a) for _ in range(4)]
+            P = K.Points(wide, sigma, handle=h, stream=b)
+            y = K.krr_kernel_mvp_points(P, Q, 1e-3, stream=b)
+            torch.cuda.synchronize()
+            P.close()
+            assert torch.equal(y, want_Q)
+            assert all(torch.equal(v, want_q) for v in ys)
