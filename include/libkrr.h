@@ -27,7 +27,9 @@
  *             The caller owns every array; the library never frees one.
  *             No array may alias another unless a function says so.
  * Streams:    `stream` is a cudaStream_t passed as void* (NULL = legacy
- *             default stream).  All device work of a call runs on it.
+ *             default stream).  All device work of a call runs on it, or on a
+ *             stream of the library's own that forks from it and joins it
+ *             again within the call (never while `stream` is being captured).
  * Handle:     a krr_handle binds to the device that is current when it is
  *             created and owns the device workspace (grown on demand, freed by
  *             krr_destroy).  A handle is not thread-safe: use one per host

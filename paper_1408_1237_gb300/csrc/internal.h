@@ -108,9 +108,14 @@ struct Ctx {
   cudaStream_t work = nullptr;
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
   // a second stream inside one product, forked from and joined to the
-  // product's own stream by ev_fork / ev_join (null: no fork).  Sub-contexts
-  // and point sets use their handle's: calls on a handle do not overlap on the host.
+  // product's own stream by ev_fork / ev_join (null: no fork; can_fork).
+  // Sub-contexts use their handle's.  A point set has its own, made by its
+  // first product that forks (lazy_aux), so that products of different point
+  // sets on different streams do not wait for each other.
   cudaStream_t aux = nullptr;
+  bool lazy_aux = false;
+  // the stream that the library itself captures (the solvers' c.work)
+  cudaStream_t captured = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   // concurrent branches of a batched solve each get a sub-context with its
   // own workspace and error word (sub-contexts own no streams or events)
@@ -263,6 +268,10 @@ constexpr double TUNE_MAX_BYTES = 1073741824.0;
 
 // Sub-context k of c (created on first use; freed with the handle).
 cudaError_t sub_context(Ctx& c, size_t k, Ctx** out);
+// Whether a product on st may fork onto c.aux.  Not while a caller captures
+// st: aux would belong to that capture until it ends, and a product on another
+// stream that forked meanwhile would break it.
+bool can_fork(Ctx& c, cudaStream_t st);
 void release_context(Ctx& c);
 
 // Points prepared while one of these is on are sorted in Morton order.

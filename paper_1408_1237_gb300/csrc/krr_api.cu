@@ -130,6 +130,7 @@ cudaError_t sub_context(Ctx& c, size_t k, Ctx** out) {
     s->aux = c.aux;
     s->ev_fork = c.ev_fork;
     s->ev_join = c.ev_join;
+    s->captured = c.work;
     s->h_counts = c.h_counts;  // whoever writes the words waits for them
     cudaError_t e = cudaMalloc(&s->d_err, sizeof(int));
     if (!e) e = cudaMemset(s->d_err, 0, sizeof(int));
@@ -141,6 +142,26 @@ cudaError_t sub_context(Ctx& c, size_t k, Ctx** out) {
   }
   *out = c.subs[k];
   return cudaSuccess;
+}
+
+bool can_fork(Ctx& c, cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (cs != cudaStreamCaptureStatusNone) return c.aux && st == c.captured;
+  if (!c.aux && c.lazy_aux) {
+    c.lazy_aux = false;
+    cudaError_t e = cudaEventCreateWithFlags(&c.ev_fork, cudaEventDisableTiming);
+    if (!e) e = cudaEventCreateWithFlags(&c.ev_join, cudaEventDisableTiming);
+    if (!e) e = cudaStreamCreateWithFlags(&c.aux, cudaStreamNonBlocking);
+    if (e) {
+      cudaGetLastError();
+      c.aux = nullptr;  // no fork
+    }
+  }
+  return c.aux != nullptr;
 }
 
 void release_context(Ctx& c) {
@@ -294,6 +315,7 @@ krr_status krr_create(krr_handle* out) {
   if (!e) e = cudaEventCreate(&c.ev0);
   if (!e) e = cudaEventCreate(&c.ev1);
   if (!e) e = cudaStreamCreateWithFlags(&c.work, cudaStreamNonBlocking);
+  c.captured = c.work;
   if (!e) e = cudaEventCreateWithFlags(&c.ev_in, cudaEventDisableTiming);
   if (!e) e = cudaEventCreateWithFlags(&c.ev_out, cudaEventDisableTiming);
   if (!e) e = cudaStreamCreateWithFlags(&c.aux, cudaStreamNonBlocking);
@@ -551,6 +573,9 @@ static void free_points(krr_points_s* pts) {
   release_context(pts->ctx);
   pts->ctx.ws.release_all();
   cudaFree(pts->ctx.d_err);
+  if (pts->ctx.aux) cudaStreamDestroy(pts->ctx.aux);
+  for (cudaEvent_t ev : {pts->ctx.ev_fork, pts->ctx.ev_join})
+    if (ev) cudaEventDestroy(ev);
   delete pts;
 }
 
@@ -576,9 +601,7 @@ krr_status krr_points_create(krr_handle h, const float* X, int64_t N, int d, flo
   Ctx& pc = pts->ctx;
   pc.device = c.device;
   pc.num_sms = c.num_sms;
-  pc.aux = c.aux;
-  pc.ev_fork = c.ev_fork;
-  pc.ev_join = c.ev_join;
+  pc.lazy_aux = true;
   copy_product_options(pc, c);
   cudaError_t e = cudaMalloc(&pc.d_err, sizeof(int));
   if (!e) e = cudaMemsetAsync(pc.d_err, 0, sizeof(int), st);

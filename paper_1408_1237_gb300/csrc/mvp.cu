@@ -1436,13 +1436,13 @@ cudaError_t mvp_multi_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, c
   p.fac = (float*)fac;
   cudaEvent_t pev1 = prof_begin(c, Tp, Sp, st);
   // Both kinds of super-block present and one kernel's CTAs fewer than the SMs:
-  // the direct-form kernel runs beside the other on a forked stream, joined
-  // before the finalize (2,000 points, 11 columns: 11.1 and 12.5 us one after
-  // the other; the gradient of 2,000 points 359 -> 242 ms).  Both are sized to
-  // fill the chip at larger sizes, where nothing would overlap.  The tuner
-  // times the kernels one after the other.
-  const bool fork = c.aux && !c.tuning && nexp > 0 && Tp.nsb > nexp &&
-                    std::min((Tp.nsb - nexp) * pd.splits, nexp * pt.splits) <= c.num_sms;
+  // the direct-form kernel runs beside the other on a forked stream (where
+  // can_fork allows one), joined before the finalize (2,000 points, 11 columns:
+  // 11.1 and 12.5 us one after the other; the gradient of 2,000 points 359 ->
+  // 242 ms).  Both are sized to fill the chip at larger sizes, where nothing
+  // would overlap.  The tuner times the kernels one after the other.
+  const bool fork = !c.tuning && nexp > 0 && Tp.nsb > nexp &&
+                    std::min((Tp.nsb - nexp) * pd.splits, nexp * pt.splits) <= c.num_sms && can_fork(c, st);
   struct Join {
     Ctx& c;
     cudaStream_t st;

@@ -143,3 +143,63 @@ def test_point_sets_created_beside_products_on_another_stream(K):
             P.close()
             assert torch.equal(y, want_Q)
             assert all(torch.equal(v, want_q) for v in ys)
+
+
+@pytest.mark.parametrize("other", [True, False])
+def test_product_beside_the_capture_of_another(K, other):
+    """A product that runs both kinds of block side by side (11 columns at 2,000
+    points) while the caller captures one on another stream, over another point
+    set or the same one: neither disturbs the other, and the replays agree."""
+    import torch
+    rng = np.random.default_rng(31)
+    X, Q = _dev(rng.random((2000, 4)).astype(np.float32)), _dev(rng.standard_normal((11, 2000)).astype(np.float32))
+    sigma, gamma = 0.2, 1e-2
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    with K.Handle() as h:
+        want = K.krr_kernel_mvp(X, Q, sigma, gamma, handle=h)
+        P1 = K.Points(X, sigma, handle=h)
+        P2 = K.Points(X, sigma, handle=h) if other else P1
+        outs = [torch.empty_like(Q) for _ in range(4)]
+        for P in (P1, P2):
+            K.krr_kernel_mvp_points(P, Q, gamma, out=outs[0])  # the shape's first call allocates
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=a):
+            K.krr_kernel_mvp_points(P1, Q, gamma, out=outs[0], stream=a)
+            K.krr_kernel_mvp_points(P2, Q, gamma, out=outs[1], stream=b)
+            K.krr_kernel_mvp_points(P1, Q, gamma, out=outs[2], stream=a)
+        torch.cuda.synchronize()
+        outs[0].zero_()
+        g.replay()
+        K.krr_kernel_mvp_points(P2, Q, gamma, out=outs[3]) if other else outs[3].copy_(want)
+        torch.cuda.synchronize()
+        assert all(torch.equal(y, want) for y in outs)
+        P1.close()
+        if other:
+            P2.close()
+
+
+def test_products_of_two_point_sets_do_not_wait_for_each_other(K):
+    """A product whose stream is held up does not hold up another point set's."""
+    import torch
+    rng = np.random.default_rng(32)
+    X, Q = _dev(rng.random((2000, 4)).astype(np.float32)), _dev(rng.standard_normal((11, 2000)).astype(np.float32))
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    with K.Handle() as h:
+        P1, P2 = K.Points(X, 0.2, handle=h), K.Points(X, 0.2, handle=h)
+        outs = [torch.empty_like(Q) for _ in range(2)]
+        for P, y in zip((P1, P2), outs):
+            K.krr_kernel_mvp_points(P, Q, 1e-2, out=y)
+        torch.cuda.synchronize()
+        done = torch.cuda.Event()
+        with torch.cuda.stream(a):
+            torch.cuda._sleep(400_000_000)  # about 0.2 s
+        K.krr_kernel_mvp_points(P1, Q, 1e-2, out=outs[0], stream=a)
+        K.krr_kernel_mvp_points(P2, Q, 1e-2, out=outs[1], stream=b)
+        done.record(b)
+        done.synchronize()
+        held = not a.query()
+        torch.cuda.synchronize()
+        assert held and torch.equal(outs[0], outs[1])
+        P1.close()
+        P2.close()
