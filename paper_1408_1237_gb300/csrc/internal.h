@@ -148,6 +148,10 @@ struct Ctx {
   bool direct_tensor = true;
   // sort points in Morton order (MortonScope)
   bool morton = false;
+  // products keep the bits that krr_mll_grad's results hang on (set while it
+  // runs): dL/dlog sigma cancels by 1e4 and more, and solutions that differ by
+  // 6e-9 move it by up to 2e-6
+  bool keep_bits = false;
   // kernel function of every product and solve (KRR_KERNEL_*, krr_set_option)
   int kernel_family = 0;
   // autotuning of the products' source splits (KRR_OPT_AUTOTUNE): the first
@@ -177,7 +181,7 @@ struct Ctx {
 
 // Product shape key of the autotuner: kind ("mvp", "fine" for MvpOut::fine, or
 // "acc"), sizes, columns,
-// precision, kernel family and the planning context.
+// precision, kernel family, the planning context, and whether krr_mll_grad asks.
 std::string tune_key(const Ctx& c, const char* kind, const PointsDev& Tp, const PointsDev& Sp, int m,
                      int prec);
 // The tuned split scale of a shape (1 when untuned).

@@ -59,9 +59,9 @@ void Workspace::release_prefix(const std::string& prefix) {
 std::string tune_key(const Ctx& c, const char* kind, const PointsDev& Tp, const PointsDev& Sp, int m,
                      int prec) {
   char buf[256];
-  snprintf(buf, sizeof(buf), "%s|%lld|%lld|%d|%d|%d|%d|%d|%d|%lld|%lld", kind, (long long)Tp.N,
+  snprintf(buf, sizeof(buf), "%s|%lld|%lld|%d|%d|%d|%d|%d|%d|%lld|%lld%s", kind, (long long)Tp.N,
            (long long)Sp.N, Tp.d, Tp.kfam, m, prec, c.plan_slots, c.tcgen05_auto ? 3 : c.use_tcgen05 ? c.tcgen05_kind : 0,
-           (long long)Tp.h_nexp, (long long)Tp.h_sb_nexp);
+           (long long)Tp.h_nexp, (long long)Tp.h_sb_nexp, c.keep_bits ? "|g" : "");
   return buf;
 }
 

@@ -344,6 +344,11 @@ extern "C" krr_status krr_mll_grad(krr_handle h, const float* X, int64_t N, int 
   // the solutions); the adjoint takes the direct form for every pair, so the
   // order costs it nothing
   MortonScope order(c, true);
+  struct KeepBits {
+    Ctx& c;
+    explicit KeepBits(Ctx& cc) : c(cc) { c.keep_bits = true; }
+    ~KeepBits() { c.keep_bits = false; }
+  } keep_bits(c);
   const int P = n_probes, nrhs = 1 + P, ncols = 2 * P + 1;
   float *dXin, *dy, *ddX = nullptr;
   bool sX, sy, sdX = false;

@@ -988,9 +988,9 @@ cudaError_t autotune_mvp(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, int m
     c.tune_variant[key] = v;
     float ms;
     if ((e = time_it(ms))) break;
-    // (a solver's choice by 8%: its products' last bits depend on it, and runs of
-    // one kernel at small sizes differ by 2%)
-    if (best_v_ms < 0.f || ms < (tcgen05_only ? 0.92f : 0.98f) * best_v_ms) {
+    // (krr_mll_grad's choice by 8%, in keys of its own: its results hang on the
+    // last bits of the products, and runs of one kernel at small sizes differ by 2%)
+    if (best_v_ms < 0.f || ms < (tcgen05_only && c.keep_bits ? 0.92f : 0.98f) * best_v_ms) {
       best_v_ms = ms;
       best_v = v;
     }

@@ -697,7 +697,7 @@ cudaError_t autotune_acc(Ctx& c, const PointsDev& P, int ncols, cudaStream_t st,
   for (double s : TUNE_SCALES) {
     c.tune_cache[key] = s;
     if (s > 1.0 &&
-        8.0 * acc_plan(P, c.num_sms, c.plan_slots, ncols, s, !c.morton).splits * ncols * (double)P.Npad > TUNE_MAX_BYTES)
+        8.0 * acc_plan(P, c.num_sms, c.plan_slots, ncols, s, !c.keep_bits).splits * ncols * (double)P.Npad > TUNE_MAX_BYTES)
       continue;
     auto run = [&]() {
       return mvp_acc_launch(c, P, (const float*)qv, (const float*)qv, 0.f, 0.0, nullptr, 1.0, (double*)yv,
@@ -737,7 +737,7 @@ cudaError_t mvp_acc_reserve(Ctx& c, const PointsDev& P, cudaStream_t st, int nco
     if (te) return te;
   }
   TuneScope scope(c, tuned_scale(c, key));
-  const AccPlan pl = acc_plan(P, c.num_sms, c.plan_slots, ncols, c.split_scale, !c.morton);
+  const AccPlan pl = acc_plan(P, c.num_sms, c.plan_slots, ncols, c.split_scale, !c.keep_bits);
   void* v;
   cudaError_t e;
   if ((e = c.ws.get("acc.part", sizeof(double) * ncols * pl.splits * (size_t)P.Npad, &v))) return e;
@@ -780,7 +780,7 @@ cudaError_t mvp_acc_launch(Ctx& c, const PointsDev& P, const float* qh, const fl
   const double sd = std::sqrt(P.s2);
   p.k.sh = (float)sd;
   p.k.sl = (float)(sd - (double)p.k.sh);
-  const AccPlan pl = acc_plan(P, c.num_sms, c.plan_slots, ncols, c.split_scale, !c.morton);
+  const AccPlan pl = acc_plan(P, c.num_sms, c.plan_slots, ncols, c.split_scale, !c.keep_bits);
   p.tiles_per_split = pl.tiles_per_split;
   p.splits = pl.splits;
   p.sub = pl.sub;

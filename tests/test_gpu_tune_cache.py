@@ -87,3 +87,23 @@ def test_tune_cache_refuses_bad_files(K, tmp_path):
         K.krr_tune_load(good, handle=h)  # an empty cache loads
     finally:
         h.close()
+
+
+def test_gradient_keeps_its_own_kernel_choice(K, tmp_path):
+    """krr_mll_grad chooses its block solves' kernel by a wider margin than the
+    solvers do: neither takes the other's choice for one shape (a compact cloud,
+    the same counts in both orders)."""
+    rng = np.random.default_rng(12)
+    X = _dev(0.01 * rng.random((600, 4)).astype(np.float32))
+    B = _dev(rng.standard_normal((16, 600)).astype(np.float32))
+    path = tmp_path / "tune.txt"
+    keys = []
+    with K.Handle() as h:
+        opts = K.default_opts(tol=1e-4)
+        K.krr_mll_grad(X, B[0].contiguous(), 0.1, 0.5, n_probes=15, opts=opts, handle=h)
+        for _ in range(2):
+            K.krr_tune_save(path, handle=h)
+            keys.append({line.split("\t")[0] for line in path.read_text().splitlines()[1:]})
+            K.krr_fgmres_solve(X, B, 0.1, 0.5, opts=opts, handle=h)
+    mine = {k for k in keys[0] if k.endswith("|g")}
+    assert mine and {k[:-2] for k in mine} <= keys[1] - keys[0]
