@@ -184,6 +184,9 @@ struct Ctx {
 // precision, kernel family, the planning context, and whether krr_mll_grad asks.
 std::string tune_key(const Ctx& c, const char* kind, const PointsDev& Tp, const PointsDev& Sp, int m,
                      int prec);
+// Whether single-column float32 products over N points in d dimensions have
+// been tuned, for any block counts (which are in the key).
+bool shape_tuned(const Ctx& c, int64_t N, int d);
 // The tuned split scale of a shape (1 when untuned).
 inline double tuned_scale(const Ctx& c, const std::string& key) {
   const auto it = c.tune_cache.find(key);

@@ -56,13 +56,19 @@ void Workspace::release_prefix(const std::string& prefix) {
   }
 }
 
+// The part of a tuning key that is known without the block counts.
+static std::string shape_key(const Ctx& c, const char* kind, int64_t Nt, int64_t Ns, int d, int kfam, int m, int prec) {
+  char buf[256];
+  snprintf(buf, sizeof(buf), "%s|%lld|%lld|%d|%d|%d|%d|%d|%d|", kind, (long long)Nt, (long long)Ns, d, kfam, m, prec,
+           c.plan_slots, c.tcgen05_auto ? 3 : c.use_tcgen05 ? c.tcgen05_kind : 0);
+  return buf;
+}
+
 std::string tune_key(const Ctx& c, const char* kind, const PointsDev& Tp, const PointsDev& Sp, int m,
                      int prec) {
-  char buf[256];
-  snprintf(buf, sizeof(buf), "%s|%lld|%lld|%d|%d|%d|%d|%d|%d|%lld|%lld%s", kind, (long long)Tp.N,
-           (long long)Sp.N, Tp.d, Tp.kfam, m, prec, c.plan_slots, c.tcgen05_auto ? 3 : c.use_tcgen05 ? c.tcgen05_kind : 0,
-           (long long)Tp.h_nexp, (long long)Tp.h_sb_nexp, c.keep_bits ? "|g" : "");
-  return buf;
+  char buf[64];
+  snprintf(buf, sizeof(buf), "%lld|%lld%s", (long long)Tp.h_nexp, (long long)Tp.h_sb_nexp, c.keep_bits ? "|g" : "");
+  return shape_key(c, kind, Tp.N, Sp.N, Tp.d, Tp.kfam, m, prec) + buf;
 }
 
 // The product over prepared points (both krr_kernel_mvp and
@@ -112,6 +118,14 @@ cudaError_t product_prepared(Ctx& c, const PointsDev& P, const float* dQ, int m,
     if ((e = mvp_multi_launch(c, P, P, qc, mc, qc, gamma, prec, o, st))) return e;
   }
   return cudaSuccess;
+}
+
+bool shape_tuned(const Ctx& c, int64_t N, int d) {
+  if (c.tune_cache.empty()) return false;
+  const std::string shape = shape_key(c, "mvp", N, N, d, c.kernel_family, 1, KRR_FP32);
+  for (const auto& kv : c.tune_cache)
+    if (kv.first.compare(0, shape.size(), shape) == 0) return true;
+  return false;
 }
 
 bool can_tune(const Ctx& c, cudaStream_t st) {
@@ -535,7 +549,7 @@ krr_status krr_kernel_mvp(krr_handle h, const float* X, int64_t N, int d, float 
   // wait for the preparation (4096 points: 70 us a call
   // with it and three product launches, 52 without)
   // (a capturing stream keeps the wait, which refuses it)
-  bool counts = m != 1 || !mvp_whole_fits(c, N, padded_dim(d), prec) || !c.tune_cache.empty();
+  bool counts = m != 1 || !mvp_whole_fits(c, N, padded_dim(d), prec) || shape_tuned(c, N, d);
   if (!counts) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {

@@ -1294,8 +1294,9 @@ bool mvp_whole_fits(const Ctx& c, int64_t N, int d, krr_precision prec) {
 }
 
 cudaError_t mvp_whole_launch(Ctx& c, const PointsDev& P, const float* Q, float shift, float* Y, cudaStream_t st) {
-  // (a loaded tuning file: the key holds the block counts, so they were read)
-  TuneScope scope(c, c.tune_cache.empty() ? 1.0 : tuned_scale(c, tune_key(c, "mvp", P, P, 1, KRR_FP32)));
+  // (the key holds the block counts, which were read if the shape may be tuned)
+  TuneScope scope(c, P.counts_read && !c.tune_cache.empty() ? tuned_scale(c, tune_key(c, "mvp", P, P, 1, KRR_FP32))
+                                                            : 1.0);
   const Plan pl = f32_plan(c, P, P);
   const size_t ctas = (size_t)((P.nblk + NW - 1) / NW);
   void *part, *fac, *tick;

@@ -107,3 +107,31 @@ def test_gradient_keeps_its_own_kernel_choice(K, tmp_path):
             K.krr_fgmres_solve(X, B, 0.1, 0.5, opts=opts, handle=h)
     mine = {k for k in keys[0] if k.endswith("|g")}
     assert mine and {k[:-2] for k in mine} <= keys[1] - keys[0]
+
+
+def test_tuning_of_other_shapes_brings_no_wait(K, tmp_path):
+    """A small single-column product waits for the device only if its own shape
+    may have been tuned."""
+    import time
+    import torch
+    rng = np.random.default_rng(13)
+    X = _dev(rng.random((3000, 3)).astype(np.float32))
+    Y = _dev(rng.random((2000, 3)).astype(np.float32))
+    q, p = (_dev(rng.standard_normal(n).astype(np.float32)) for n in (3000, 2000))
+    path = tmp_path / "tune.txt"
+    with _tuned_handle(K) as h:
+        K.krr_kernel_mvp(Y, p, 0.1, 1e-3, handle=h)
+        tuned = K.krr_kernel_mvp(Y, p, 0.1, 1e-3, handle=h)
+        K.krr_tune_save(path, handle=h)
+    with K.Handle() as h:
+        want = K.krr_kernel_mvp(X, q, 0.1, 1e-3, handle=h)
+        K.krr_tune_load(path, handle=h)
+        for A, w, ref, waits in ((X, q, want, False), (Y, p, tuned, True)):
+            K.krr_kernel_mvp(A, w, 0.1, 1e-3, handle=h)
+            torch.cuda.synchronize()
+            torch.cuda._sleep(600_000_000)  # about 0.3 s
+            t0 = time.perf_counter()
+            y = K.krr_kernel_mvp(A, w, 0.1, 1e-3, handle=h)
+            held = time.perf_counter() - t0 > 0.1
+            torch.cuda.synchronize()
+            assert held == waits and torch.equal(y, ref)
