@@ -24,6 +24,7 @@ own independent problem (seeded by rank) and ranks exchange only timings.
 """
 import argparse
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -360,11 +361,14 @@ def run_libkrr(args):
     value = whole_job_rate(pairs * args.steps, world, total_s)
     launches = prof["launches"] - launches0
     kern_ms = prof["product_ms"] / max(prof["product_launches"], 1)
-    achieved = pairs / (kern_ms / 1e3) / 1e9
     # CUDA-core work per pair of the product's path (expanded form): one
     # MUFU.EX2, plus d + 1 FP32 operations when the exponent is formed on the
     # CUDA cores, or 1 (the weighted accumulate) when the tensor cores form it
     tensor_exp = prof["tensor_exponent_launches"] == prof["product_launches"] > 0
+    # that kernel leaves out source tiles of exact zeros: only the pairs it
+    # evaluates count against a peak per evaluated pair
+    evaluated = evaluated_pairs(torch, X, sigma) if tensor_exp else pairs
+    achieved = evaluated / (kern_ms / 1e3) / 1e9
     fp32_per_pair = 1 if tensor_exp else MVP_D + 1
     peak_pairs = min(ex2_rate, fp32_lanes / fp32_per_pair)
     kernel_name = ("mvp_tcx_kernel (exponent on the tensor cores) + direct-form tail"
@@ -481,8 +485,10 @@ def run_libkrr(args):
                 "unit": "Gpairs/s", "frac": achieved * 1e9 / peak_pairs,
                 "traffic": traffic_bytes(tensor_exp),
                 "kernel": kernel_name, "launch_ms": kern_ms,
-                "pairs": "all N^2; the kernel leaves out source tiles whose kernel values "
-                         "are exact zeros in its arithmetic (the sums are the same bit for bit)",
+                "pairs": "those evaluated: source tiles whose kernel values are exact zeros in "
+                         "the kernel's arithmetic are left out (the sums are the same bit for bit)",
+                "evaluated_fraction": evaluated / pairs,
+                "all_pairs_Gpairs_per_s": pairs / (kern_ms / 1e3) / 1e9,
                 "peak_source": "measured on this GPU: min(MUFU.EX2 rate, FP32 lane rate / FP32 "
                                f"operations per pair) = min({ex2_rate / 1e12:.2f}e12, "
                                f"{fp32_lanes / 1e12:.2f}e12/{fp32_per_pair})",
@@ -512,6 +518,53 @@ def run_libkrr(args):
         import torch.distributed as dist
         dist.destroy_process_group()
     return 0
+
+
+def hilbert_order(torch, X, bits):
+    """The points along the library's Hilbert curve (J. Skilling, AIP Conf.
+    Proc. 707, 2004), `bits` bits per coordinate."""
+    d = X.shape[1]
+    lo, hi = X.amin(0), X.amax(0)
+    cells = ((X - lo) / (hi - lo) * float(1 << bits)).clamp(0, (1 << bits) - 1).to(torch.int64)
+    x = list(cells.unbind(1))
+    for b in range(bits - 1, 0, -1):
+        low = (1 << b) - 1
+        for k in range(d):
+            top = ((x[k] >> b) & 1).bool()
+            t = torch.where(top, low, (x[0] ^ x[k]) & low)
+            x[0] = x[0] ^ t
+            if k > 0:
+                x[k] = torch.where(top, x[k], x[k] ^ t)
+    for k in range(1, d):
+        x[k] = x[k] ^ x[k - 1]
+    t = torch.zeros_like(x[0])
+    for b in range(bits - 1, 0, -1):
+        t = torch.where(((x[d - 1] >> b) & 1).bool(), t ^ ((1 << b) - 1), t)
+    key = torch.zeros_like(t)
+    for b in range(bits):
+        for k in range(d):
+            key |= (((x[k] ^ t) >> b) & 1) << (b * d + d - 1 - k)
+    return torch.sort(key, stable=True).indices
+
+
+def evaluated_pairs(torch, X, sigma, tile=256, cut=128.0, expanded_r2=8.0):
+    """Pairs of points that a float32 single-column product over X evaluates:
+    compact blocks of targets leave out the source tiles whose box lies so far
+    from theirs that every kernel value is below 2^-126, wide blocks take all.
+    Restates the kernel's rule on the sorted points' boxes (N a multiple of
+    the tile)."""
+    N, d = X.shape
+    s2 = 0.5 / (math.log(2.0) * sigma * sigma)
+    P = X[hilbert_order(torch, X, min(16, 30 // d))].reshape(-1, tile, d)
+    lo, hi = P.amin(1), P.amax(1)
+    c, h = 0.5 * (lo + hi), 0.5 * (hi - lo)
+    compact = s2 * (P - c[:, None]).square().sum(2).amax(1) <= expanded_r2
+    tiles = 0
+    for i in range(0, len(c), 512):
+        gap = (c[i:i + 512, None] - c).abs() - h[i:i + 512, None] - h
+        near = s2 * (gap.clamp(min=0.0).square().sum(2) - h[i:i + 512, None].square().sum(2)) <= cut
+        tiles += int((near | ~compact[i:i + 512, None]).sum())
+    return float(tiles) * tile * tile
 
 
 def traffic_bytes(tensor_exp):

@@ -43,3 +43,26 @@ def test_both_arms_report_the_same_workload():
     assert set(cfg) == {"workload", "l2", "parallelism"}
     assert "N=1048576" in cfg["workload"] and "d=3" in cfg["workload"]
     assert bench.bench_config(4)["workload"] == cfg["workload"]
+
+
+def test_evaluated_pairs_leave_out_far_tiles_of_compact_blocks_only():
+    import torch
+    g = torch.Generator().manual_seed(3)
+    near = torch.rand(512, 3, generator=g)
+    two = torch.cat([near, near + 100.0])  # two clusters of two tiles each
+    full = float(two.shape[0]) ** 2
+    assert bench.evaluated_pairs(torch, two, 2.0) == full / 2
+    assert bench.evaluated_pairs(torch, two, 200.0) == full
+    assert bench.evaluated_pairs(torch, two, 0.01) == full  # wide blocks: the direct form takes every pair
+
+
+def test_hilbert_order_visits_neighbouring_cells():
+    import itertools
+
+    import torch
+    n = 8
+    cells = torch.tensor(list(itertools.product(range(n), repeat=3)), dtype=torch.float32)
+    cells = cells[torch.randperm(len(cells), generator=torch.Generator().manual_seed(4))]
+    X = torch.cat([(cells + 0.5) / n, torch.zeros(1, 3), torch.ones(1, 3)])  # the corners set the box
+    walk = (X[bench.hilbert_order(torch, X, 3)] * n).clamp(max=n - 1).floor()
+    assert (walk[1:] - walk[:-1]).abs().sum(1).max() == 1
