@@ -677,12 +677,22 @@ struct Plan {
 // scale: the autotuner's factor on the modelled split count (1: the model);
 // setup: a CTA's fixed cost (launch, target loads, epilogue) in source tiles.
 // Without it the model prefers many splits of a tile or two to a slightly
-// longer last wave: 64 direct-form blocks and 65 tiles got 33 splits of 2
-// (16,385 points, d = 8, f16, 16 columns: 354 us, and 301 with 7 splits of 10).
-// Where a tile is long it hardly counts, and finer splits balance better
-// (Matern, 8 targets per thread, 100,003 points: 3.62 ms with 49 splits of 8
-// tiles, 3.84 with 6 of 66).
-constexpr double SETUP_F32 = 0.3;    // mvp_f32_kernel, per 1 / T (T targets per thread)
+// longer last wave; with too much of it a few long splits, whose last CTAs run
+// alone on their SMs.  Mean and worst time over a sweep of sizes and d against
+// the best of five or six setups each:
+//   mvp_f32_kernel, 33 shapes of one target per thread (1,005 to 50,568
+//   points): 0: 1.009, 1.16; 0.05: 1.004, 1.04; 0.3: 1.013, 1.18 (d = 8, 11,233
+//   points: 89 us with 0.05, 106 with 0.3); 30 shapes of several (set per
+//   1 / T): 0.05: 1.001, 1.01; 0.3: 1.010, 1.12 (d = 8, 114,300 points 5.06 and
+//   5.68 ms);
+//   mvp_tcx_kernel, 16 shapes: 0: 1.020, 1.11; 0.1: 1.030, 1.26 (d = 1, 101,491
+//   points 804 and 1011 us); 0.3: 1.017, 1.26; but 468 us with 0 and 388 with 0.1
+//   for 98,869 targets of 29,204 sources, d = 1, whose splits of two tiles hold
+//   little but exact zeros;
+//   mvp_tc_kernel, 20 shapes: 0: 1.027, 1.39; 0.3: 1.005, 1.07; 0.6: 1.010, 1.15;
+//   mvp_dirtc_kernel, 20 shapes: 0: 1.026, 1.29; 0.5: 1.001, 1.01; 2: 1.010,
+//   1.09 (16,385 points, d = 8, f16, 16 columns: 303 us with 0, 250 with 0.5).
+constexpr double SETUP_F32 = 0.05;   // mvp_f32_kernel, per 1 / T (T targets per thread)
 constexpr double SETUP_TCX = 0.1;    // mvp_tcx_kernel
 constexpr double SETUP_MULTI = 0.3;  // mvp_tc_kernel, mvp_umx_kernel
 constexpr double SETUP_DIRTC = 0.5;  // mvp_dirtc_kernel (512 threads, one CTA per SM)
