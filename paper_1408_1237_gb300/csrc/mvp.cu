@@ -112,18 +112,26 @@ __device__ __forceinline__ void transform_tile(const float* __restrict__ rs, flo
   }
 }
 
-// Sources per unrolled step are 4 times this: with one target per thread the
-// instruction chains of several sources have to fill the pipes.
+// Sources per unrolled step are 4 U.  With one target per thread a single wave
+// of CTAs is bound by latency: the instruction chains of many sources fill the
+// pipes (U = 8; 12,288 points, d = 2: 45.5 us, 61.6 with U = 2).  In several waves
+// of short CTAs more of them on an SM do that (58 registers with U = 2, four
+// CTAs; 104 with U = 8, two): 16,384 points, d = 2 74.5 us with U = 2 and 81.3
+// with 8, 32,000 points 253 and 274, d = 4 365 and 397; from d = 5 on shared
+// memory allows no more CTAs (32,000 points 455 and 451; so too for the whole
+// product in one launch from d = 4 on: 16,384 points 117 and 113).  U = 2 in one wave would also
+// let an early start pile four CTAs on some SMs (24,576 points, d = 2: 298 us,
+// 163 with U = 8).
 template <int T>
-constexpr int f32_unroll() { return T == 1 ? 8 : 2; }
+constexpr int one_wave_unroll() { return T == 1 ? 8 : 2; }
 
-template <int D, int T>
+template <int D, int T, int U>
 __device__ __forceinline__ void compute_expanded(const float* __restrict__ cb,
                                                  const float2 (&tx)[T][D], float2 (&acc)[T]) {
   const float* cX = cb;
   const float* cB = cb + D * TS;
   const float* cQ = cb + (D + 1) * TS;
-#pragma unroll f32_unroll<T>()
+#pragma unroll U
   for (int j = 0; j < TS; j += 4) {
     float4 xk[D];
 #pragma unroll
@@ -158,7 +166,7 @@ __device__ __forceinline__ float matern32_value(float r2, float s) {
 }
 
 // KF: pair function, 0 = Gaussian 2^(-s^2 r^2), 1 = Matern 3/2 (s = sqrt(3)/h).
-template <int D, int T, int KF>
+template <int D, int T, int KF, int U>
 __device__ __forceinline__ void compute_direct(const float* __restrict__ cb,
                                                const float2 (&tx)[T][D], float2 (&acc)[T],
                                                float s2, float s) {
@@ -166,7 +174,7 @@ __device__ __forceinline__ void compute_direct(const float* __restrict__ cb,
   const float* cQ = cb + (D + 1) * TS;
   const float2 ns2 = make_float2(-s2, -s2);
   const float2 sv = make_float2(s, s), nl2e = make_float2(-kLog2e, -kLog2e);
-#pragma unroll f32_unroll<T>()
+#pragma unroll U
   for (int j = 0; j < TS; j += 4) {
     float4 xk[D];
 #pragma unroll
@@ -209,7 +217,7 @@ __device__ __forceinline__ void compute_direct(const float* __restrict__ cb,
 }
 
 // WHOLE: the whole product of a small point set (MvpParams::q_orig)
-template <int D, int T, int KF, bool WHOLE>
+template <int D, int T, int KF, bool WHOLE, int U>
 __global__ void __launch_bounds__(NT, 2) mvp_f32_kernel(const MvpParams p) {
   constexpr int RS = raw_stages<D>();
   constexpr uint32_t kRawFloats = (D + 1) * TS;
@@ -326,9 +334,9 @@ __global__ void __launch_bounds__(NT, 2) mvp_f32_kernel(const MvpParams p) {
       transform_tile<D>(raw + (r % RS) * kRawFloats, wbuf, ctr, p.s, expanded);
       __syncwarp();
       if (expanded)
-        compute_expanded<D, T>(wbuf, tx, acc);
+        compute_expanded<D, T, U>(wbuf, tx, acc);
       else
-        compute_direct<D, T, KF>(wbuf, tx, acc, s2, p.s);
+        compute_direct<D, T, KF, U>(wbuf, tx, acc, s2, p.s);
 #pragma unroll
       for (int u = 0; u < T; ++u) {
         kahan_add(sum[u], comp[u], acc[u].x + acc[u].y);
@@ -609,26 +617,26 @@ constexpr size_t smem_bytes() {
 }
 
 // Dynamic shared-memory opt-in, once per kernel instance and device.
-template <int D, int T, int KF, bool WHOLE = false>
+template <int D, int T, int KF, bool WHOLE = false, int U = one_wave_unroll<T>()>
 cudaError_t set_attr() {
   static bool done[128] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 128 && done[dev]) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(mvp_f32_kernel<D, T, KF, WHOLE>,
+  cudaError_t e = cudaFuncSetAttribute(mvp_f32_kernel<D, T, KF, WHOLE, U>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem_bytes<D>());
   if (!e && dev < 128) done[dev] = true;
   return e;
 }
 
-template <int D, int T, int KF, bool WHOLE = false>
+template <int D, int T, int KF, bool WHOLE = false, int U = one_wave_unroll<T>()>
 cudaError_t launch_typed(const MvpParams& p, int splits, cudaStream_t st) {
-  cudaError_t e = set_attr<D, T, KF, WHOLE>();
+  cudaError_t e = set_attr<D, T, KF, WHOLE, U>();
   if (e) return e;
   dim3 grid((unsigned)std::max<int64_t>(1, (p.nblk - p.slot0 + NW - 1) / NW), (unsigned)splits);
-  if (p.pdl) return launch_pdl(mvp_f32_kernel<D, T, KF, WHOLE>, grid, NT, smem_bytes<D>(), st, p);
-  mvp_f32_kernel<D, T, KF, WHOLE><<<grid, NT, smem_bytes<D>(), st>>>(p); count_launch();
+  if (p.pdl) return launch_pdl(mvp_f32_kernel<D, T, KF, WHOLE, U>, grid, NT, smem_bytes<D>(), st, p);
+  mvp_f32_kernel<D, T, KF, WHOLE, U><<<grid, NT, smem_bytes<D>(), st>>>(p); count_launch();
   return cudaGetLastError();
 }
 
@@ -672,6 +680,7 @@ int large_T_of(int d) {
 struct Plan {
   int splits = 1;
   int tiles_per_split = 1;
+  bool one_wave = true;  // every CTA is resident at once (in the slots planned for)
 };
 
 // scale: the autotuner's factor on the modelled split count (1: the model);
@@ -705,6 +714,7 @@ Plan make_plan(int64_t nblk, int ntiles, int num_sms, int plan_slots, double sca
     splits = std::max(1, std::min({(int)std::lround(splits * scale), ntiles, 256}));
   pl.tiles_per_split = (ntiles + splits - 1) / splits;
   pl.splits = (ntiles + pl.tiles_per_split - 1) / pl.tiles_per_split;
+  pl.one_wave = ctas * pl.splits <= slots;
   return pl;
 }
 
@@ -712,7 +722,12 @@ template <int D, int KF = 0>
 cudaError_t attrs_T(int T) {
   constexpr int TL = large_T<D>();
   if (T == TL) return set_attr<D, TL, KF>();
-  if (T == 1) return set_attr<D, 1, KF>();
+  if (T == 1) {
+    cudaError_t e = set_attr<D, 1, KF>();
+    if constexpr (D <= 4)
+      if (!e) e = set_attr<D, 1, KF, false, 2>();
+    return e;
+  }
   return cudaErrorNotSupported;
 }
 
@@ -720,6 +735,10 @@ template <int D, int KF = 0>
 cudaError_t dispatch_T(MvpParams p, int T, const Plan& pl, cudaStream_t st) {
   constexpr int TL = large_T<D>();
   p.tiles_per_split = pl.tiles_per_split;
+  if constexpr (D <= 3)
+    if (T == 1 && !pl.one_wave && p.q_orig) return launch_typed<D, 1, KF, true, 2>(p, pl.splits, st);
+  if constexpr (D <= 4)
+    if (T == 1 && !pl.one_wave && !p.q_orig) return launch_typed<D, 1, KF, false, 2>(p, pl.splits, st);
   if (p.q_orig) return T == 1 ? launch_typed<D, 1, KF, true>(p, pl.splits, st) : cudaErrorNotSupported;
   if (T == TL) return launch_typed<D, TL, KF>(p, pl.splits, st);
   if (T == 1) return launch_typed<D, 1, KF>(p, pl.splits, st);

@@ -58,3 +58,21 @@ def test_one_launch_equals_three(K, oracle_mod, N, d, family):
     h.close()
     g.close()
 
+
+
+@pytest.mark.parametrize("N,d", [(12288, 2), (12289, 2), (16384, 4), (20000, 3), (24576, 2), (24577, 4), (32001, 1)])
+@pytest.mark.parametrize("family", [0, 1])
+def test_products_in_one_and_in_several_waves(K, oracle_mod, N, d, family):
+    """Both depths of unrolling of the one-target kernel, against the oracle on
+    sampled rows."""
+    X, q = _data(N, d, N + d)
+    sigma, gamma = 0.1 * d ** 0.5, 1e-2
+    with K.Handle() as h:
+        K.krr_set_option(K.KRR_OPT_KERNEL, family, handle=h)
+        y = K.krr_kernel_mvp(X, q, sigma, gamma, handle=h).cpu().numpy()
+    rows = np.random.default_rng(N).choice(N, 64, replace=False)
+    X64, q64 = X.cpu().numpy().astype(np.float64), q.cpu().numpy().astype(np.float64)
+    kernel = "matern32" if family else "gaussian"
+    ref = oracle_mod.mvp(X64, q64, f32(sigma), f32(gamma), rows=rows, kernel=kernel)
+    scale = oracle_mod.mvp(X64, np.abs(q64), f32(sigma), f32(gamma), rows=rows, kernel=kernel)
+    assert np.max(np.abs(y[rows] - ref) / scale) <= 1e-5
