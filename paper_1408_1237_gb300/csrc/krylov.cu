@@ -233,8 +233,8 @@ __global__ void cg_p_kernel(KState* S0, const float* __restrict__ r, float* __re
   KRR_GRID_LOOP(i) p[co + i] = fmaf(b, p[co + i], r[co + i]);
 }
 
-// ---- a whole CG step after the product's partial sums, in one launch for Np <=
-// STEP_MAX_NP: M p from the sums, alpha = rho / p.Mp, z += alpha p, r -= alpha
+// ---- a whole CG step after the product's partial sums, in one launch for small
+// problems (fused_step): M p from the sums, alpha = rho / p.Mp, z += alpha p, r -= alpha
 // M p, rho' = |r|^2, beta = rho'/rho, the continuation test and p = r + beta p.
 // One cluster of STEP_CL CTAs per column: a thread keeps its R rows in
 // registers from the first phase to the last (M p is never written), and the
@@ -248,9 +248,16 @@ __global__ void cg_p_kernel(KState* S0, const float* __restrict__ r, float* __re
 // 1 / rho is formed meanwhile, which leaves one division on the path.
 constexpr int STEP_CL = 8;
 constexpr int STEP_T = 256;
-// above, 8 SMs per column take longer over the FP64 sums than the three
-// kernels on all SMs (16384 rows: about 4 us of FP64 at 8 splits)
-constexpr int64_t STEP_MAX_NP = 16384;
+// Above, 8 SMs per column take longer over the FP64 sums than the three kernels
+// on all SMs: a row costs one addition per source split and a few more, two per
+// clock and SM.  Time per CG step against the three kernels (d = 2): one column
+// 12.3 and 25.0 us at 2,000 points, 34.0 and 42.5 at 8,192, 61.1 and 64.3 at
+// 12,288, but 105 and 87 at 14,336 (56 splits), 111 and 99 at 16,384; 4 columns
+// 101 and 95 at 16,384; from 5 columns on, whose products take more of the
+// step, it gains up to there (5 columns 131 and 135 us at 16,000 points, 16
+// columns 63.8 and 74.8 at 8,192, 135 and 142 at 16,384).
+constexpr int64_t STEP_MAX_NP = 16384, STEP_MAX_NP_FEW = 12288;
+constexpr int STEP_MANY_COLS = 5;
 constexpr int CG_UNROLL = 4;  // CG steps per turn of the graph's loop
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
@@ -1104,6 +1111,8 @@ struct Solver {
     cfg.attrs = at;
     cfg.numAttrs = 1;
   }
+  // Whether a CG step runs as the product and cg_step_kernel.
+  bool fused_step() const { return Np <= (mc >= STEP_MANY_COLS ? STEP_MAX_NP : STEP_MAX_NP_FEW); }
   template <typename F>
   F rows_of(F k1, F k2, F k4, F k8) const {
     const int64_t rows = (Np + STEP_CL * STEP_T - 1) / (STEP_CL * STEP_T);
@@ -1132,7 +1141,7 @@ struct Solver {
   // for every column whose CG continues
   cudaError_t cg_iteration() {
     MvpOut o;
-    if (Np <= STEP_MAX_NP) {
+    if (fused_step()) {
       o.active = &G->cg_any;
       o.finish = cg_step;
       o.finish_arg = this;
@@ -1328,7 +1337,7 @@ cudaError_t fill_restart_body(Solver& s, cudaGraph_t rbody, double tol_stop) {
   // several predicated CG steps per turn of the loop: a step of a small problem
   // costs less than the loop's own turn (a step after the last column has
   // stopped only reads its flag)
-  const int unroll = s.Np <= STEP_MAX_NP ? CG_UNROLL : 1;
+  const int unroll = s.fused_step() ? CG_UNROLL : 1;
   if ((e = capture_into(s.st, cbody, [&]() -> cudaError_t {
          cudaError_t ee = cudaSuccess;
          for (int k = 0; k < unroll && !ee; ++k) ee = s.cg_iteration();

@@ -45,3 +45,8 @@ def test_solve_at_the_row_boundaries(K, oracle_mod, N, m):
         b = B[c].astype(np.float64)
         r = b - oracle_mod.mvp(X64, sols[0][c], f32(sigma), f32(gamma))
         assert np.linalg.norm(r) <= 1e-6 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("N,m", [(12288, 1), (12289, 1), (12288, 4), (12289, 4), (12289, 5), (16384, 5), (16385, 5)])
+def test_steps_at_the_boundaries_of_few_and_many_columns(K, oracle_mod, N, m):
+    test_solve_at_the_row_boundaries(K, oracle_mod, N, m)
