@@ -150,6 +150,7 @@ typedef enum {
      *     solvers (block, batched and gradient solves) instead time 0 and 1
      *     once per product shape when they reserve it (a few products,
      *     before any graph capture) and keep the faster.
+     * krr_kernel_mvp_rect in float32 takes 0 whatever the value.
      * Same results to the float32 bar (and the reduced-precision bars).  On
      * GB300, 16 columns at 2^20 points in float32: 65 / 84 / 546 ms for
      * 1 / 0 / 2 (2 visits every tile of pairs).  Other values:
@@ -295,7 +296,10 @@ krr_status krr_points_destroy(krr_handle h, krr_points P);
 /* Prediction product of Eq. GPR_mean / Eq. Kriging:
  *     Y[t,c] = sum_j exp(-|xt_t - xs_j|^2 / (2 sigma^2)) Q[j,c]
  * Xt: Nt x d targets, Xs: Ns x d sources, Q: Ns x m, Y: Nt x m (no diagonal
- * term).  Asynchronous on device arrays. */
+ * term).  Weights may have any size, and targets may lie away from all sources:
+ * in float32, up to 8 dimensions, the error stays below 1e-5 of
+ * sum_j |Q_jc| K_hat_tj up to six widths outside the cloud.  Asynchronous on device arrays, but for the waits for the two
+ * preparations. */
 krr_status krr_kernel_mvp_rect(krr_handle h, const float* Xt, int64_t Nt,
                                const float* Xs, int64_t Ns, int d, float sigma,
                                const float* Q, int m, float* Y,
@@ -442,7 +446,9 @@ typedef struct {
                                rest ran the CUDA-core kernels                  */
 } krr_profile;
 /* Start (enable != 0) or stop timing the fast-product kernel on h; resets the
- * timed list.  Timing adds two event records per product launch. */
+ * timed list.  Timing adds two event records per product launch, and small
+ * single-column products run as gather, product kernel and finalize instead of
+ * one launch (the same results). */
 krr_status krr_profile_enable(krr_handle h, int enable);
 /* Fill *out, waiting for the recorded events, and reset the timed list. */
 krr_status krr_profile_read(krr_handle h, krr_profile* out);

@@ -95,7 +95,7 @@ def test_targets_away_from_all_sources(K, oracle_mod, m, d, sigma):
         got = errors(oracle_mod, Xt, Xs, Q[:3], K.krr_kernel_mvp_rect(Xtd, Xsd, Qd, sigma)[:3].cpu().numpy(), sigma)
         alone = np.stack([K.krr_kernel_mvp_rect(Xtd, Xsd, Qd[c].contiguous(), sigma).cpu().numpy() for c in range(3)])
         one = errors(oracle_mod, Xt, Xs, Q[:3], alone, sigma)
-        assert got.max() <= (TOL if out <= 6 else TOL_FAR), (out, got, one)
+        assert max(got.max(), one.max()) <= (TOL if out <= 6 else TOL_FAR), (out, got, one)
         if out <= 3:
             assert (got <= one + SPLIT).all(), (out, got, one)
 
