@@ -43,10 +43,10 @@ METRIC = "Gaussian kernel MVP Gpairs/s; FGMRES time-to-1e-6 residual vs plain FP
 # taken on.
 TRAFFIC = {"sources": {"paper_1408_1237_gb300/csrc/mvp.cu": "9775246cbc799cc4467e0840befecdb000cb45d1"},
            "bytes": 22374656 + 83717888}
-# the same for the tensor-core exponent path (mvp_tcx_kernel + direct-form tail)
-TRAFFIC_TCX = {"sources": {"paper_1408_1237_gb300/csrc/mvp.cu": "c97b0b9bbaaeb44ef0f54387704d2631a12ca666",
-                           "paper_1408_1237_gb300/csrc/mvp_tc.cu": "56d5c2079577a7fb0c3bb0e0a57e1d21f79255e6"},
-               "bytes": 22713600 + 92372480 + 17144576 + 0}
+# the same for the tensor-core exponent path (mvp_tcx_kernel and the finalize)
+TRAFFIC_TCX = {"sources": {"paper_1408_1237_gb300/csrc/mvp.cu": "48b9585d1fe437b3dad74683979d1bc3a9d1546b",
+                           "paper_1408_1237_gb300/csrc/mvp_tc.cu": "c8b84af5d8de51372f312d2b5d51c374f53ed734"},
+               "bytes": 17029376 + 164608 + 46171648 + 0}
 MVP_N, MVP_D = 1 << 20, 3
 
 

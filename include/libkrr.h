@@ -152,7 +152,7 @@ typedef enum {
      *     before any graph capture) and keep the faster.
      * krr_kernel_mvp_rect in float32 takes 0 whatever the value.
      * Same results to the float32 bar (and the reduced-precision bars).  On
-     * GB300, 16 columns at 2^20 points in float32: 65 / 84 / 546 ms for
+     * GB300, 16 columns at 2^20 points in float32: 65 / 77 / 546 ms for
      * 1 / 0 / 2 (2 visits every tile of pairs).  Other values:
      * KRR_ERR_INVALID_ARG. */
     KRR_OPT_TCGEN05 = 1,

@@ -1311,9 +1311,11 @@ cudaError_t mvp_launch(Ctx& c, const PointsDev& Tp, const PointsDev& Sp, const f
 }
 
 // One launch instead of gather, product and finalize.  With few points the
-// three are launch latency and the host's three calls (4,096 prepared points:
-// 27 us a product and 19 with one); each CTA gathers the weights of its
-// tiles itself, which above WHOLE_MAX_N costs more than the gather.
+// three are launch latency and the host's three calls; each CTA gathers the
+// weights of its tiles itself, which grows with the splits.  d = 3, one launch
+// and three: krr_kernel_mvp at 4,096, 12,288, 16,384 points 54 and 66, 100 and
+// 112, 144 and 153 us; prepared points as a graph 12.3 and 14.7, 54.7 and 58.5,
+// 97.8 and 96.2, and at 32,768 351 and 342 us.
 constexpr int64_t WHOLE_MAX_N = 16384;
 
 bool mvp_whole_fits(const Ctx& c, int64_t N, int d, krr_precision prec) {
