@@ -110,3 +110,42 @@ def test_infinite_weight_stays_in_its_column(K):
     z = K.krr_kernel_mvp_rect(*dev, Q, 0.2)
     torch.cuda.synchronize()
     assert torch.equal(y[1:], z[1:]) and not torch.isfinite(z[0]).any()
+
+
+@pytest.mark.parametrize("family", ["gaussian", "matern32"])
+@pytest.mark.parametrize("d,width", [(2, 0.2), (5, 0.5), (12, 1.2), (33, 1.4)])
+@pytest.mark.parametrize("m", [2, 5, 17])
+def test_columns_together_and_alone(K, oracle_mod, m, d, width, family):
+    """Every route of several columns (two kernel families, d above 8, one and
+    two passes) against the oracle and the same columns alone."""
+    import torch
+    Xt, Xs, rng = _clouds(d, 1237, 1411, m + d)
+    Q = rng.standard_normal((m, 1411)).astype(np.float32)
+    dev = [torch.from_numpy(a).cuda() for a in (Xt, Xs, Q)]
+    with K.Handle() as h:
+        K.krr_set_option(K.KRR_OPT_KERNEL, {"gaussian": K.KRR_KERNEL_GAUSSIAN, "matern32": K.KRR_KERNEL_MATERN32}[family],
+                         handle=h)
+        y = K.krr_kernel_mvp_rect(*dev, width, handle=h).cpu().numpy()
+        for c in {0, m - 1}:
+            alone = K.krr_kernel_mvp_rect(dev[0], dev[1], dev[2][c].contiguous(), width, handle=h).cpu().numpy()
+            q = Q[c].astype(np.float64)
+            args = (Xt.astype(np.float64), Xs.astype(np.float64))
+            ref = oracle_mod.mvp_rect(*args, q, f32(width), kernel=family)
+            scale = oracle_mod.mvp_rect(*args, np.abs(q), f32(width), kernel=family)
+            got, one = (np.max(np.abs(v - ref) / scale) for v in (y[c], alone))
+            assert one <= TOL and got <= min(TOL, one + SPLIT), (got, one)
+
+
+def test_many_targets_take_the_same_kernels(K, oracle_mod):
+    """From 131,072 targets and 9 columns on the automatic choice of the square
+    products is a tcgen05 kernel."""
+    import torch
+    Xt, Xs, rng = _clouds(3, 131073, 1501, 8)
+    Q = rng.standard_normal((9, 1501)).astype(np.float32)
+    dev = [torch.from_numpy(a).cuda() for a in (Xt, Xs, Q)]
+    y = K.krr_kernel_mvp_rect(*dev, 0.1)
+    with K.Handle() as h:
+        K.krr_set_option(K.KRR_OPT_TCGEN05, 0, handle=h)
+        assert torch.equal(K.krr_kernel_mvp_rect(*dev, 0.1, handle=h), y)
+    rows = rng.choice(131073, 64, replace=False)
+    assert errors(oracle_mod, Xt[rows], Xs, Q, y[:, torch.from_numpy(rows).cuda()].cpu().numpy(), 0.1).max() <= TOL
