@@ -238,7 +238,10 @@ krr_status krr_set_option(krr_handle h, int option, int value);
  * (tensor cores for compact target blocks).
  * prec: KRR_FP32 (max relative error per element, against the FP64 sum
  * scaled by sum_j |Q_jc| K_hat_ij + gamma |Q_ic|, below 1e-5) or KRR_BF16 /
- * KRR_FP16 (reduced-precision kernel values, float32 accumulation).  In 16
+ * KRR_FP16 (reduced-precision kernel values, float32 accumulation).  Several
+ * columns (m >= 2) hold the weights that compact blocks meet as f16, in float32
+ * as f16 hi + lo: a column's weights should be below 65504 in size and the
+ * largest of them above 1e-3 (scale others by a power of two).  In 16
  * bits, up to 8 dimensions and under the Gaussian kernel, the points are sorted
  * in Morton instead of Hilbert order: which targets share a block decides the
  * form their kernel values are rounded in.

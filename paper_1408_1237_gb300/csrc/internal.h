@@ -298,7 +298,7 @@ struct MortonScope {
 // 70,001 in d = 2 moved by 3.1e-4 (relative), bf16 by 2.5e-3, and those of
 // 16,385 normal points in d = 8 by up to 4e-5 through the two targets that are
 // alone in the last block.  Products in 16 bits therefore keep the Morton
-// order, and with it their results; float32 products differ by 4e-7 at most.
+// order, and with it their results; float32 products moved by 1e-6 at most.
 inline bool order_decides(int kernel_family, int d, krr_precision prec) {
   return prec != KRR_FP32 && kernel_family == KRR_KERNEL_GAUSSIAN && d <= 8;
 }
